@@ -531,6 +531,12 @@ int hol_tune(hol_ctx* ctx, int n_rhs, int* best_k, int* best_warps, int* best_ve
  *                       (rows in bands over several warps) where it is
  *                       built (L = 4-18 even, 24, 28, 32) unless this is 0,
  *                       else the shared-memory kernel
+ *   "resident_cg"       plain CG (no preconditioner, checkerboard) with a
+ *                       right-hand side's whole state on chip, one cluster of
+ *                       thread blocks each and one launch per solve, where it
+ *                       fits (FP32 iterations: N Ltau up to about 230,000 at
+ *                       L = 32; FP64: small systems); 0: the iteration
+ *                       kernels below (0/1, default 1)
  *   "persistent_cg"     plain mixed CG chunks in one cooperative launch (0/1)
  *   "pdl"               programmatic dependent launch of the CG iteration
  *                       kernels: each may be scheduled while its predecessor
@@ -580,8 +586,8 @@ int hol_tune(hol_ctx* ctx, int n_rhs, int* best_k, int* best_warps, int* best_ve
  * Every solver variant certifies convergence by the FP64 true residual;
  * iteration counts may differ by a few percent between them.
  * A context with the exact propagator (HOL_KINETIC_EXACT) keeps layout 0 and
- * refuses any other layout and kpm_registers, persistent_cg, fused_cg and
- * merged_cg set to 1 (those kernels are checkerboard only).
+ * refuses any other layout and kpm_registers, resident_cg, persistent_cg,
+ * fused_cg and merged_cg set to 1 (those kernels are checkerboard only).
  * Returns HOL_EINVAL for an unknown name or a value out of range (HOL_ECUDA
  * when an allocation fails).
  */

@@ -849,6 +849,35 @@ static int cg_run(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_c
 }
 
 
+// The plain CG on chip (resident.cuh): one launch, results read back once.
+static int cg_run_resident(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_opts* o,
+                           int* iters, double* resid, cudaStream_t s)
+{
+    const long R = c->p.max_rhs;
+    const DcgState d = dcg_state(c);
+    timer_start(c, KT_OPERATOR, s);
+    if (int rc = resident_enqueue(c, b, v, n_rhs, o, s)) return rc;
+    timer_stop(c, KT_OPERATOR, s);
+    double* tres = c->hbuf;
+    int* ih = c->hflag;   // it, since, done, rstate [R each], g
+    HOL_CUDA(cudaMemcpyAsync(tres, d.tres, n_rhs * sizeof(double), cudaMemcpyDeviceToHost, s));
+    HOL_CUDA(cudaMemcpyAsync(ih, d.it, (size_t)(4 * R + DCG_COUNT) * sizeof(int),
+                             cudaMemcpyDeviceToHost, s));
+    HOL_CUDA(cudaStreamSynchronize(s));
+    int all = 1;
+    for (int k = 0; k < n_rhs; ++k) {
+        if (iters) iters[k] = ih[k];
+        if (resid) resid[k] = tres[k];
+        all &= ih[2 * R + k];
+    }
+    const int* g = ih + 4 * R;
+    if (g[DCG_ERR])
+        return set_error(HOL_ENUMERIC, "cg_solve: non-finite residual (rhs %d)", g[DCG_ERR_RHS]);
+    if (!all)
+        return set_error(HOL_ENOTCONV, "cg_solve: not converged within %d iterations", o->max_iter);
+    return HOL_OK;
+}
+
 // Mixed plain CG with one fused kernel per iteration (k_cg_fused in
 // matvec.cu): the vector update of iteration i and the operator of
 // iteration i + 1 share one pass over the vectors, and beta comes from the
@@ -1462,6 +1491,7 @@ int cg_run_dev(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_o
         return set_error(HOL_EINVAL, "graph solve: needs the two-kernel CG iteration (fused_cg, "
                                      "merged_cg and persistent_cg off)");
     if (pc && (rc = precond_check_shape(c))) return rc;
+    if (resident_ok(c, o, n_rhs)) return resident_enqueue(c, b, v, n_rhs, o, s);
 
     double* r64 = c->v64a;
     double* p64[2] = {c->v64b, c->v64c};
@@ -1672,5 +1702,7 @@ extern "C" int cg_solve(hol_ctx* c, const double* b, double* v, int n_rhs, const
         return cg_run_fused(c, b, v, n_rhs, o, iters, resid, (cudaStream_t)stream);
     if (c->merged && o->prec == HOL_F32 && !o->precond)
         return cg_run_merged(c, b, v, n_rhs, o, iters, resid, (cudaStream_t)stream);
+    if (resident_ok(c, o, n_rhs))
+        return cg_run_resident(c, b, v, n_rhs, o, iters, resid, (cudaStream_t)stream);
     return cg_run(c, b, v, n_rhs, o, iters, resid, (cudaStream_t)stream);
 }

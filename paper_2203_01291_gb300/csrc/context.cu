@@ -295,6 +295,7 @@ extern "C" int hol_create(const hol_params* p, hol_ctx** out)
     c->persist = 0;
     c->merged = 0;
     c->fused = 0;
+    c->resident = c->exact ? 0 : 1;
     c->pdl = 1;
     c->kpm_a1 = 1.0;
     c->kpm_a2 = 1.0;
@@ -372,7 +373,7 @@ extern "C" int hol_create(const hol_params* p, hol_ctx** out)
     ALLOC(c->cbuf1, c->cbuf_len * sizeof(double2));
 #undef ALLOC
     if (cudaMallocHost((void**)&c->hbuf, 16 * R * sizeof(double)) != cudaSuccess ||
-        cudaMallocHost((void**)&c->hflag, 4 * R * sizeof(int)) != cudaSuccess) {
+        cudaMallocHost((void**)&c->hflag, (4 * R + DCG_COUNT) * sizeof(int)) != cudaSuccess) {
         free_ctx(c);
         return set_error(HOL_ENOMEM, "hol_create: pinned host allocation failed");
     }
@@ -571,6 +572,10 @@ extern "C" int hol_set_option(hol_ctx* c, const char* name, int value)
         if (value && c->exact)
             return set_error(HOL_EINVAL, "hol_set_option: persistent_cg is checkerboard only");
         c->persist = value ? 1 : 0;
+    } else if (is("resident_cg")) {
+        if (value && c->exact)
+            return set_error(HOL_EINVAL, "hol_set_option: resident_cg is checkerboard only");
+        c->resident = value ? 1 : 0;
     } else if (is("pdl")) {
         c->pdl = value ? 1 : 0;
     } else if (is("fused_pc_update")) {
@@ -621,6 +626,7 @@ extern "C" int hol_get_option(const hol_ctx* c, const char* name, int* value)
     else if (is("persistent_cg")) *value = c->persist;
     else if (is("merged_cg")) *value = c->merged;
     else if (is("fused_cg")) *value = c->fused;
+    else if (is("resident_cg")) *value = c->resident;
     else if (is("pdl")) *value = c->pdl;
     else if (is("scalar_handoff")) *value = c->handoff;
     else if (is("kpm_queue")) *value = c->kpm_queue;

@@ -149,6 +149,18 @@ struct KpmPlan {
     double2* coef;       // [T/2][max_np] complex c_m(omega)
 };
 
+struct ResArgs;
+// Launch plan of the on-chip CG for n_rhs right-hand sides (resident.cu).
+struct ResPlan {
+    int n_rhs;           // 0: not yet planned
+    int cs, clusters;    // blocks per cluster; clusters launched
+    int warps, k, slots; // warps per block, slices per lane group, most slices per block
+    int tm_cols;         // tensor-memory columns (0: none used)
+    size_t smem;
+    double us;           // modelled time of one iteration of all right-hand sides
+    void (*fn)(ResArgs); // null: no plan fits
+};
+
 }  // namespace hol
 
 struct hol_ctx {
@@ -248,6 +260,8 @@ struct hol_ctx {
     int* kpm_q;          // its work queue [2] (next problem, finished blocks; zero between launches)
     double kpm_a1, kpm_a2;   // constants of the Chebyshev order heuristic (1, 1 by default)
     int pc_fuse;             // PCG: vector update fused into the preconditioner's transform
+    int resident;            // launch option "resident_cg": plain CG with its state on chip
+    hol::ResPlan res_plan[2];    // its plan for the last n_rhs, by precision (resident.cu)
 };
 
 namespace hol {
@@ -371,11 +385,12 @@ struct DcgState {
     int* it;
     int* since;
     int* done;
+    int* rstate;     // on-chip CG: ready / running / done (resident.cuh)
     int* g;
 };
 inline size_t dcg_bytes(long R)
 {
-    return (size_t)(4 * R) * sizeof(double) + (size_t)(3 * R + DCG_COUNT) * sizeof(int);
+    return (size_t)(4 * R) * sizeof(double) + (size_t)(4 * R + DCG_COUNT) * sizeof(int);
 }
 inline DcgState dcg_state(const hol_ctx* c)
 {
@@ -389,7 +404,8 @@ inline DcgState dcg_state(const hol_ctx* c)
     d.it = ib;
     d.since = ib + R;
     d.done = ib + 2 * R;
-    d.g = ib + 3 * R;
+    d.rstate = ib + 3 * R;
+    d.g = ib + 4 * R;
     return d;
 }
 // Graph-capturable CG: the solve of cg_solve (the same kernels and the same
@@ -400,6 +416,13 @@ inline DcgState dcg_state(const hol_ctx* c)
 // in dcg_state(c) and v.
 int cg_run_dev(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_opts* o,
                cudaStream_t s);
+// The plain CG with its state on chip (resident.cu): whether the context and
+// options take it for n_rhs right-hand sides, and one solve enqueued on s
+// (capturable; results in dcg_state(c)).
+const ResPlan& resident_plan(hol_ctx* c, int prec, int n_rhs);
+bool resident_ok(hol_ctx* c, const hol_cg_opts* o, int n_rhs);
+int resident_enqueue(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_opts* o,
+                     cudaStream_t s);
 // Conditional nodes in a capturing stream: cond_handle creates a handle in the
 // graph being captured on s (capture the kernel that sets it next);
 // cond_node appends the node after the stream's current dependencies, makes
