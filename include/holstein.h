@@ -518,18 +518,15 @@ int hol_tune(hol_ctx* ctx, int n_rhs, int* best_k, int* best_warps, int* best_ve
  *                       slice per warp and slices_per_group (<= 8) warps per
  *                       block exchanging the tau neighbours in shared memory
  *                       (L == 32)
- *   "kpm_registers"     FP32 KPM with the slice in registers: 0 off
- *                       (shared-memory kernel), 1 four columns per lane
- *                       (L = 16 or 32), 2 two columns per lane (L = 16 or
- *                       32: twice the warps per problem, half the work per
- *                       lane on the chain of Bbar applies), 3 the lane
- *                       layout (any L: one lane per column, the rows in
- *                       registers, the real and imaginary parts in two lane
- *                       groups). 1 and 2 fall back to the shared-memory
- *                       kernel for other L. Default 2 at L = 32, 3
- *                       otherwise. The FP64 KPM uses the banded lane layout
- *                       (rows in bands over several warps) where it is
- *                       built (L = 4-18 even, 24, 28, 32) unless this is 0,
+ *   "kpm_registers"     Chebyshev kernels of the preconditioner: 4 (default)
+ *                       column-pair strips in registers, FP32 and FP64, any L,
+ *                       each problem over as many warps as its longest series
+ *                       needs; the older kernels: 0 shared memory (both
+ *                       precisions), 1 / 2 FP32 four / two columns per lane
+ *                       (L = 16 or 32, else shared memory), 3 FP32 lane layout
+ *                       (one lane per column, the real and imaginary parts in
+ *                       two lane groups); with 1..3 FP64 uses the banded lane
+ *                       layout where it is built (L = 4-18 even, 24, 28, 32),
  *                       else the shared-memory kernel
  *   "resident_cg"       plain CG (no preconditioner, checkerboard) with a
  *                       right-hand side's whole state on chip, one cluster of

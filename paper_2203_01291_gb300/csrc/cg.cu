@@ -533,7 +533,7 @@ static int cg_run(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_c
     const int pq_n = c->T / c->mv_k;
     int pstride64 = 0, pq_n64 = 0;   // the FP64 CG's M keeps its own grouping
     fp64_cg_geom(c, n_rhs, &pstride64, &pq_n64);
-    const int dz_n = pc ? precond_tiles(c, prec) : nb2;   // partial count of r.z
+    const int dz_n = pc ? precond_tiles(c, prec, n_rhs) : nb2;   // partial count of r.z
     // PCG: the vector update inside the preconditioner's forward transform;
     // the r.r estimate then has one partial per transform tile
     const bool fuse_pc = pc && c->pc_fuse;
@@ -1476,7 +1476,7 @@ int cg_run_dev(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_o
     const int pq_n = c->T / c->mv_k;
     int pstride64 = 0, pq_n64 = 0;   // the FP64 CG's M keeps its own grouping
     fp64_cg_geom(c, n_rhs, &pstride64, &pq_n64);
-    const int dz_n = pc ? precond_tiles(c, mixed ? HOL_F32 : HOL_F64) : nb2;
+    const int dz_n = pc ? precond_tiles(c, mixed ? HOL_F32 : HOL_F64, n_rhs) : nb2;
     const bool fuse_pc = pc && c->pc_fuse;   // as in cg_run
     const int est_n = fuse_pc ? dz_n : nb2;
     int* act_d = c->mask;

@@ -285,13 +285,8 @@ extern "C" int hol_create(const hol_params* p, hol_ctx** out)
     c->mv_k = (c->T % 4 == 0 && c->T >= 8) ? 2 : 1;
     c->mv_warps = 4;
     c->mv_vec = c->exact ? 0 : 1;
-    // register KPM: two columns per lane at L = 32 (measured 0.126 against
-    // 0.149 ms for P^{-1} P^{-T} on 16 rhs; 47 us against 58 us for the lane
-    // layout on 2 rhs at Ltau = 200), the lane layout (one lane per column,
-    // real and imaginary parts in two lane groups) for every other L (at
-    // L = 16, Ltau = 160, 2 rhs: 25.3 us against 29.0 us for four columns
-    // per lane)
-    c->kpm_reg = c->exact ? 0 : (c->L == 32 ? 2 : 3);
+    // Chebyshev kernels of kpm.cu (measured there against the older layouts)
+    c->kpm_reg = c->exact ? 0 : 4;
     c->persist = 0;
     c->merged = 0;
     c->fused = 0;
@@ -565,8 +560,8 @@ extern "C" int hol_set_option(hol_ctx* c, const char* name, int value)
     } else if (is("kpm_registers")) {
         if (value && c->exact)
             return set_error(HOL_EINVAL, "hol_set_option: kpm_registers is checkerboard only");
-        if (value < 0 || value > 3)
-            return set_error(HOL_EINVAL, "hol_set_option: kpm_registers must be 0, 1, 2 or 3");
+        if (value < 0 || value > 4)
+            return set_error(HOL_EINVAL, "hol_set_option: kpm_registers must be 0..4");
         c->kpm_reg = value;
     } else if (is("persistent_cg")) {
         if (value && c->exact)

@@ -70,6 +70,62 @@ __device__ __forceinline__ C cmi(C a)
     return r;
 }
 
+// Length-RAD DFT of a[] in place (root[e] = exp(-2 pi i e / RAD)). Odd lengths
+// pair the inputs r and RAD - r: with s = a_r + a_{RAD-r}, d = a_r - a_{RAD-r}
+// the outputs q and RAD - q are (a_0 + sum cos s) -/+ i (sum sin d), a third of
+// the products of the plain sums (radix 5: 36 operations instead of 120).
+template <typename R, int RAD>
+__device__ __forceinline__ void dft_small(typename Cx<R>::T2 (&a)[RAD],
+                                          const typename Cx<R>::T2 (&root)[RAD])
+{
+    using C2 = typename Cx<R>::T2;
+    if constexpr (RAD == 2) {
+        const C2 x = a[0], y = a[1];
+        a[0] = cadd(x, y);
+        a[1] = csub(x, y);
+    } else if constexpr (RAD == 4) {
+        const C2 s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
+        const C2 s13 = cadd(a[1], a[3]), d13 = cmi(csub(a[1], a[3]));
+        a[0] = cadd(s02, s13);
+        a[1] = cadd(d02, d13);
+        a[2] = csub(s02, s13);
+        a[3] = csub(d02, d13);
+    } else {
+        constexpr int HF = (RAD - 1) / 2;
+        C2 s[HF], d[HF];
+#pragma unroll
+        for (int r = 1; r <= HF; ++r) {
+            s[r - 1] = cadd(a[r], a[RAD - r]);
+            d[r - 1] = csub(a[r], a[RAD - r]);
+        }
+        const C2 a0 = a[0];
+#pragma unroll
+        for (int r = 0; r < HF; ++r) a[0] = cadd(a[0], s[r]);
+#pragma unroll
+        for (int q = 1; q <= HF; ++q) {
+            C2 re = a0, im;
+#pragma unroll
+            for (int r = 1; r <= HF; ++r) {
+                const C2 w = root[(r * q) % RAD];   // (cos, -sin)
+                re.x = fma(w.x, s[r - 1].x, re.x);
+                re.y = fma(w.x, s[r - 1].y, re.y);
+                if (r == 1) {
+                    im.x = w.y * d[0].x;
+                    im.y = w.y * d[0].y;
+                } else {
+                    im.x = fma(w.y, d[r - 1].x, im.x);
+                    im.y = fma(w.y, d[r - 1].y, im.y);
+                }
+            }
+            // re + i im with im = -(sum sin d)
+            a[q].x = re.x - im.y;
+            a[q].y = re.y + im.x;
+            a[RAD - q].x = re.x + im.y;
+            a[RAD - q].y = re.y - im.x;
+        }
+    }
+}
+
 // One Stockham pass of radix RAD over TS columns: in[tau][c] -> out[.][c].
 // Butterfly j (0 <= j < T/RAD) with k = j mod Ns reads in[j + r T/RAD],
 // scales input r by exp(-2 pi i r k / (Ns RAD)), takes the length-RAD DFT
@@ -94,38 +150,16 @@ __device__ void stockham_pass(const typename Cx<R>::T2* __restrict__ in,
     for (; j < nb; j += sj) {
         C2 a[RAD];
         a[0] = in[j * TS + c];
-        if (k > 0) {
-            const C2 w1 = w2[2L * k * tstep];
-            C2 wr = w1;
+        // twiddles from the table: powers of one cost two products each more
 #pragma unroll
-            for (int r = 1; r < RAD; ++r) {
-                a[r] = cmul(in[(j + r * nb) * TS + c], wr);
-                if (r + 1 < RAD) wr = cmul(wr, w1);
-            }
-        } else {
-#pragma unroll
-            for (int r = 1; r < RAD; ++r) a[r] = in[(j + r * nb) * TS + c];
+        for (int r = 1; r < RAD; ++r) {
+            const C2 v = in[(j + r * nb) * TS + c];
+            a[r] = k > 0 ? cmul(v, w2[2L * r * k * tstep]) : v;
         }
+        dft_small<R, RAD>(a, root);
         const int ob = jb * Ns * RAD + k;
-        if (RAD == 2) {
-            out[ob * TS + c] = cadd(a[0], a[1]);
-            out[(ob + Ns) * TS + c] = csub(a[0], a[1]);
-        } else if (RAD == 4) {
-            const C2 s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
-            const C2 s13 = cadd(a[1], a[3]), d13 = cmi(csub(a[1], a[3]));
-            out[ob * TS + c] = cadd(s02, s13);
-            out[(ob + Ns) * TS + c] = cadd(d02, d13);
-            out[(ob + 2 * Ns) * TS + c] = csub(s02, s13);
-            out[(ob + 3 * Ns) * TS + c] = csub(d02, d13);
-        } else {
 #pragma unroll
-            for (int q = 0; q < RAD; ++q) {
-                C2 s = a[0];
-#pragma unroll
-                for (int r = 1; r < RAD; ++r) s = cadd(s, cmul(a[r], root[(r * q) % RAD]));
-                out[(ob + q * Ns) * TS + c] = s;
-            }
-        }
+        for (int q = 0; q < RAD; ++q) out[(ob + q * Ns) * TS + c] = a[q];
         k += sk;
         jb += sjb;
         if (k >= Ns) {
@@ -209,38 +243,15 @@ __device__ __forceinline__ void stockham_pass_ct(const typename Cx<R>::T2* __res
         const int k = j % Ns, jb = j / Ns;
         C2 a[RAD];
         a[0] = in[j * TS + c];
-        if (Ns > 1 && k > 0) {
-            const C2 w1 = w2[2 * k * tstep];
-            C2 wr = w1;
 #pragma unroll
-            for (int r = 1; r < RAD; ++r) {
-                a[r] = cmul(in[(j + r * nb) * TS + c], wr);
-                if (r + 1 < RAD) wr = cmul(wr, w1);
-            }
-        } else {
-#pragma unroll
-            for (int r = 1; r < RAD; ++r) a[r] = in[(j + r * nb) * TS + c];
+        for (int r = 1; r < RAD; ++r) {
+            const C2 v = in[(j + r * nb) * TS + c];
+            a[r] = (Ns > 1 && k > 0) ? cmul(v, w2[2 * r * k * tstep]) : v;
         }
+        dft_small<R, RAD>(a, root);
         const int ob = jb * Ns * RAD + k;
-        if constexpr (RAD == 2) {
-            out[ob * TS + c] = cadd(a[0], a[1]);
-            out[(ob + Ns) * TS + c] = csub(a[0], a[1]);
-        } else if constexpr (RAD == 4) {
-            const C2 s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
-            const C2 s13 = cadd(a[1], a[3]), d13 = cmi(csub(a[1], a[3]));
-            out[ob * TS + c] = cadd(s02, s13);
-            out[(ob + Ns) * TS + c] = cadd(d02, d13);
-            out[(ob + 2 * Ns) * TS + c] = csub(s02, s13);
-            out[(ob + 3 * Ns) * TS + c] = csub(d02, d13);
-        } else {
 #pragma unroll
-            for (int q = 0; q < RAD; ++q) {
-                C2 sum = a[0];
-#pragma unroll
-                for (int r = 1; r < RAD; ++r) sum = cadd(sum, cmul(a[r], root[(r * q) % RAD]));
-                out[(ob + q * Ns) * TS + c] = sum;
-            }
-        }
+        for (int q = 0; q < RAD; ++q) out[(ob + q * Ns) * TS + c] = a[q];
     }
 }
 

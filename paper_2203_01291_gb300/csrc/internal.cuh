@@ -519,7 +519,7 @@ int elementwise_blocks(const hol_ctx* c, int n_rhs);
 
 // preconditioner (precond.cu). mode bit 0: P^{-T} part, bit 1: P^{-1} part
 // (both: P^{-1} P^{-T}). rdot/dot_part (nullable): partial sums of out . rdot
-// per (rhs, tile) at stride kRedStride, precond_tiles(c, prec) per rhs.
+// per (rhs, tile) at stride kRedStride, precond_tiles(c, prec, n_rhs) per rhs.
 int precond_alloc(hol_ctx* c);
 int leapfrog_alloc(hol_ctx* c);
 // Parts of one HMC trajectory (leapfrog.cu) replayed by the captured batch
@@ -543,7 +543,11 @@ int measure_run(hol_ctx* c, const double* xi, int n_rv, const hol_cg_opts* opts,
 int measure_prepare(hol_ctx* c);
 int measure_alloc(hol_ctx* c);
 int precond_check_shape(const hol_ctx* c);
-int precond_tiles(const hol_ctx* c, int prec);
+// Chebyshev kernels of one preconditioner application (kpm.cu), half spectra
+// [rhs][T/2][N] in and out; mode as precond_apply_impl
+int kpm_strip(const hol_ctx* c, const float2* in, float2* out, int n_rhs, int mode, cudaStream_t s);
+int kpm_pair(const hol_ctx* c, const double2* in, double2* out, int n_rhs, int mode, cudaStream_t s);
+int precond_tiles(const hol_ctx* c, int prec, int n_rhs);
 int precond_apply_impl(hol_ctx* c, int prec, const void* v, void* out, int n_rhs, int mode,
                        const void* rdot, double* dot_part, cudaStream_t s);
 

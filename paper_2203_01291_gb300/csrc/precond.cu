@@ -23,6 +23,9 @@
 //   k_tau_fwd     twisted DFT along tau, tiles of TS sites x T slices in
 //                 shared memory, Stockham mixed-radix passes (radix 4,2,3,5,7).
 //   k_tau_fwd_upd the same with the PCG vector update fused into its loads.
+//   kpm.cu        the Chebyshev series kernels used by default; the ones below
+//                 serve the launch option kpm_registers 0..3 and the exact
+//                 propagator:
 //   k_kpm_reg     FP32, L = 16, 32: one (omega, rhs) problem per block, two
 //                 rows and two or four complex columns per lane.
 //   k_kpm_lane    FP32, any L: lane = column, rows in registers, the real and
@@ -1244,20 +1247,23 @@ __global__ void k_kpm_coeffs(const double* __restrict__ scal, int T, int max_np,
     }
 }
 
-// Sites per tau-transform tile: 32 (FP32) / 16 (FP64) on the largest lattice;
-// 8 below it, so that a small lattice with few right-hand sides still spreads
-// over many blocks (N = 256 and 2 rhs: 64 blocks instead of 16).
-constexpr int kSmallTile = 8;
-int tile_sites(const hol_ctx* c, int prec)
+// Sites per tau-transform tile. A block's chain (loads, passes, stores) is what
+// a transform takes, so the tile is the smaller of two while that leaves at most
+// about eight blocks per multiprocessor: 8 or 16 sites in FP32 (16 rhs of L =
+// 32, Ltau = 200: forward / inverse 11.1 / 13.0 us with 16 sites, 12.1 / 15.4
+// with 32), 4
+// or 8 in FP64 (one sector per row segment), where smaller blocks spread the
+// arithmetic over the FP64 pipes of more multiprocessors.
+int tile_sites(const hol_ctx* c, int prec, int n_rhs)
 {
-    if (c->N < 1024) return kSmallTile;
-    return prec == HOL_F64 ? 16 : 32;
+    const int small = prec == HOL_F64 ? 4 : 8;
+    return (long)c->N * n_rhs <= 8L * small * c->sms ? small : 2 * small;
 }
 
-size_t fft_smem(const hol_ctx* c, int prec)
+size_t fft_smem(const hol_ctx* c, int prec, int ts)
 {
     const size_t cs = prec == HOL_F64 ? sizeof(double2) : sizeof(float2);
-    return 2 * (size_t)c->T * (tile_sites(c, prec) / 2) * cs;   // two sites per column
+    return 2 * (size_t)c->T * (ts / 2) * cs;   // two sites per column
 }
 
 template <typename R, int L>
@@ -1365,8 +1371,8 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
     using C2 = typename Cx<R>::T2;
     const int prec = sizeof(R) == 8 ? HOL_F64 : HOL_F32;
     const RadixPlan plan = plan_of(c->T);
-    const int TS = tile_sites(c, prec);
-    const size_t sm = fft_smem(c, prec);
+    const int TS = tile_sites(c, prec, n_rhs);
+    const size_t sm = fft_smem(c, prec, TS);
     const dim3 gf(ceil_div(c->N, TS), n_rhs);
     const C2* w2 = reinterpret_cast<const C2*>(prec == HOL_F64 ? (const void*)c->tw64
                                                                 : (const void*)c->tw32);
@@ -1374,7 +1380,7 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
     C2* h1 = reinterpret_cast<C2*>(c->cbuf1);
     int rc;
     // the configured lengths get transforms specialised at compile time
-    constexpr int TSW = sizeof(R) == 8 ? 16 : 32;   // tile_sites on the largest lattice
+    constexpr int TSS = sizeof(R) == 8 ? 4 : 8;   // tile_sites' two choices
     using FwdK = void (*)(const R*, C2*, const C2*, int, int, int, RadixPlan, R);
     using FwdU = void (*)(R*, C2*, const C2*, int, int, int, RadixPlan, R, PcUpdK<R>);
     using InvK = void (*)(const C2*, R*, const C2*, int, int, int, RadixPlan, R, const R*, double*);
@@ -1383,14 +1389,14 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
     InvK inv = k_tau_inv<R>;
 #define HOL_TAU_CT(TT)                                    \
     case TT:                                              \
-        if (TS == TSW) {                                  \
-            fwd = k_tau_fwd<R, TT, TSW>;                  \
-            fwdu = k_tau_fwd_upd<R, TT, TSW>;             \
-            inv = k_tau_inv<R, TT, TSW>;                  \
-        } else if (TS == kSmallTile) {                    \
-            fwd = k_tau_fwd<R, TT, kSmallTile>;           \
-            fwdu = k_tau_fwd_upd<R, TT, kSmallTile>;      \
-            inv = k_tau_inv<R, TT, kSmallTile>;           \
+        if (TS == TSS) {                                  \
+            fwd = k_tau_fwd<R, TT, TSS>;                  \
+            fwdu = k_tau_fwd_upd<R, TT, TSS>;             \
+            inv = k_tau_inv<R, TT, TSS>;                  \
+        } else {                                          \
+            fwd = k_tau_fwd<R, TT, 2 * TSS>;              \
+            fwdu = k_tau_fwd_upd<R, TT, 2 * TSS>;         \
+            inv = k_tau_inv<R, TT, 2 * TSS>;              \
         }                                                 \
         break;
     switch (c->T) {
@@ -1456,6 +1462,11 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
             if (rc) return rc;
             HOL_CHECK_LAUNCH("k_kpm_reg");
             done = true;
+        } else if (c->kpm_reg == 4 && !c->exact) {
+            rc = kpm_strip(c, reinterpret_cast<const float2*>(h0), reinterpret_cast<float2*>(h1),
+                           n_rhs, mode, s);
+            if (rc) return rc;
+            done = true;
         } else if (c->kpm_reg == 3 && !c->exact) {
             rc = run_kpm_lane<float>(c, reinterpret_cast<const float2*>(h0),
                                      reinterpret_cast<float2*>(h1), n_rhs, ka.Th, ka.max_np,
@@ -1469,7 +1480,12 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
         // SMSP's share of the FP64 pipe and measured slower than the
         // shared-memory kernel, 602 against 325 us on the L = 16,
         // Ltau = 160 trajectory's 2 rhs)
-        if (c->kpm_reg != 0 && !c->exact && kpm_band_ok(c->L)) {
+        if (c->kpm_reg == 4 && !c->exact) {
+            rc = kpm_pair(c, reinterpret_cast<const double2*>(h0), reinterpret_cast<double2*>(h1),
+                          n_rhs, mode, s);
+            if (rc) return rc;
+            done = true;
+        } else if (c->kpm_reg != 0 && !c->exact && kpm_band_ok(c->L)) {
             rc = run_kpm_band(c, reinterpret_cast<const double2*>(h0),
                               reinterpret_cast<double2*>(h1), n_rhs, ka.Th, ka.max_np, mode, s);
             if (rc) return rc;
@@ -1493,13 +1509,16 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
 
 }  // namespace
 
-int precond_tiles(const hol_ctx* c, int prec) { return ceil_div(c->N, tile_sites(c, prec)); }
+int precond_tiles(const hol_ctx* c, int prec, int n_rhs)
+{
+    return ceil_div(c->N, tile_sites(c, prec, n_rhs));
+}
 
 int precond_check_shape(const hol_ctx* c)
 {
     const RadixPlan p = plan_of(c->T);
     if (p.n < 0) return set_error(HOL_EINVAL, "preconditioner: Ltau=%d has a prime factor > 7", c->T);
-    if (fft_smem(c, HOL_F64) > 220 * 1024)
+    if (fft_smem(c, HOL_F64, c->N < 1024 ? 8 : 16) > 220 * 1024)
         return set_error(HOL_EINVAL, "preconditioner: Ltau=%d too long for one tile", c->T);
     if (c->N > kKpmMaxE * 256) return set_error(HOL_EINVAL, "preconditioner: N too large");
     return HOL_OK;
