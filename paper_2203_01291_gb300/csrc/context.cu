@@ -74,44 +74,58 @@ int cuda_error(cudaError_t e, const char* what)
 
 namespace {
 
-// ev = cosh^4 exp(-dtau (alpha x - mu)) in FP64 and FP32 (the cosh factors
-// of the four checkerboard colours, see cb.cuh); copy of x.
-__global__ void k_expv(const double* __restrict__ x, double* __restrict__ xc,
-                       double* __restrict__ ev64, float* __restrict__ ev32, long n, double dtau,
-                       double alpha, double mu, double ch4)
+// Everything of the field but the Chebyshev plan, in one launch: the copy of x,
+// ev = cosh^4 exp(-dtau (alpha x - mu)) in FP64 and FP32 (the cosh factors of the
+// four checkerboard colours, see cb.cuh), dbar_i = (1/T) sum_tau ev (Eq.
+// (expnVbar)) and, in the block that finishes last, the norm bounds of the Bbar
+// spectrum: every checkerboard colour has eigenvalues exp(+-dtau t), so |Bbar| <=
+// max(dbar) e^{4 dtau |t|} and |Bbar^{-1}| <= e^{4 dtau |t|} / min(dbar) (the
+// stored dbar carries cosh^4, removed there). A block takes kFieldSites sites
+// (one 32-byte sector of a slice) at all T slices, its threads strided over tau,
+// and adds their sums in a fixed order. Bound by the FP64 exponentials (about
+// 4 us of the FP64 pipes for 92,160 values); as three launches with one thread
+// per site in the tau sum it took 23 us at L = 24, Ltau = 160, in one 11. The
+// count of finished blocks returns to zero; no block waits for another.
+constexpr int kFieldSites = 4;
+__global__ void __launch_bounds__(256) k_field(const double* __restrict__ x, double* __restrict__ xc,
+                                               double* __restrict__ ev64, float* __restrict__ ev32,
+                                               double* __restrict__ dbar, double* __restrict__ scal,
+                                               int* __restrict__ count, int N, int T, double dtau,
+                                               double alpha, double mu, double ch4, double g4)
 {
-    for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < n;
-         k += (long)gridDim.x * blockDim.x) {
+    __shared__ double part[256];
+    __shared__ int s_last;
+    const int si = threadIdx.x % kFieldSites, t0 = threadIdx.x / kFieldSites;
+    const int i = blockIdx.x * kFieldSites + si;          // N is a multiple of four
+    double s = 0.0;
+    for (int tau = t0; tau < T; tau += 256 / kFieldSites) {
+        const long k = (long)tau * N + i;
         const double xv = x[k];
         const double e = ch4 * exp(-dtau * (alpha * xv - mu));
         xc[k] = xv;
         ev64[k] = e;
         ev32[k] = (float)e;
+        s += e;
     }
-}
-
-// dbar_i = (1/T) sum_tau expV[tau][i] (Eq. (expnVbar)); one thread per site.
-__global__ void k_dbar(const double* __restrict__ ev, double* __restrict__ dbar, int N, int T)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    double s = 0.0;
-    for (int tau = 0; tau < T; ++tau) s += ev[(long)tau * N + i];
-    dbar[i] = s / T;
-}
-
-// Norm bounds of the Bbar spectrum: every checkerboard colour has
-// eigenvalues exp(+-dtau t), so |Bbar| <= max(dbar) e^{4 dtau |t|} and
-// |Bbar^{-1}| <= e^{4 dtau |t|} / min(dbar), dbar of Eq. (expnVbar) (the
-// stored dbar carries the factor cosh^4, removed here). One block.
-__global__ void k_bounds(const double* __restrict__ dbar, int N, double g4, double ch4,
-                         double* __restrict__ scal)
-{
-    __shared__ double smin[32], smax[32];
+    part[threadIdx.x] = s;
+    __syncthreads();
+    for (int n = 128; n >= kFieldSites; n >>= 1) {
+        if (threadIdx.x < n) part[threadIdx.x] += part[threadIdx.x + n];
+        __syncthreads();
+    }
+    if (threadIdx.x < kFieldSites) dbar[i] = part[threadIdx.x] / T;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(count, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    __shared__ double smin[8], smax[8];
     double lo = 1e300, hi = -1e300;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        lo = fmin(lo, dbar[i]);
-        hi = fmax(hi, dbar[i]);
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+        const double d = __ldcg(dbar + k);
+        lo = fmin(lo, d);
+        hi = fmax(hi, d);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -125,12 +139,13 @@ __global__ void k_bounds(const double* __restrict__ dbar, int N, double g4, doub
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
+        for (int k = 1; k < 8; ++k) {
             lo = fmin(lo, smin[k]);
             hi = fmax(hi, smax[k]);
         }
         scal[S_BMIN] = lo / ch4 / g4;
         scal[S_BMAX] = hi / ch4 * g4;
+        *count = 0;
     }
 }
 
@@ -151,6 +166,10 @@ void free_ctx(hol_ctx* c)
     if (c->beta_now) cudaFree(c->beta_now);
     if (c->beta_cnt) cudaFree(c->beta_cnt);
     if (c->kpm_q) cudaFree(c->kpm_q);
+    if (c->field_cnt) cudaFree(c->field_cnt);
+    if (c->kpm.coef32) cudaFree(c->kpm.coef32);
+    if (c->kpm.dk64) cudaFree(c->kpm.dk64);
+    if (c->kpm.dk32) cudaFree(c->kpm.dk32);
     for (cudaStream_t cs : c->cap_s)
         if (cs) cudaStreamDestroy(cs);
     timer_free(c->timer);
@@ -353,9 +372,11 @@ extern "C" int hol_create(const hol_params* p, hol_ctx** out)
     ALLOC(c->beta_now, R * sizeof(double));
     ALLOC(c->beta_cnt, R * sizeof(int));
     ALLOC(c->kpm_q, 2 * sizeof(int));
+    ALLOC(c->field_cnt, 2 * sizeof(int));
     if (cudaMemset(c->alpha_cnt, 0, R * sizeof(int)) != cudaSuccess ||
         cudaMemset(c->beta_cnt, 0, R * sizeof(int)) != cudaSuccess ||
-        cudaMemset(c->kpm_q, 0, 2 * sizeof(int)) != cudaSuccess) {
+        cudaMemset(c->kpm_q, 0, 2 * sizeof(int)) != cudaSuccess ||
+        cudaMemset(c->field_cnt, 0, 2 * sizeof(int)) != cudaSuccess) {
         free_ctx(c);
         return set_error(HOL_ECUDA, "hol_create: memset");
     }
@@ -404,15 +425,10 @@ extern "C" int hol_set_field(hol_ctx* c, const double* x, void* stream)
     if (!c || !x) return set_error(HOL_EINVAL, "hol_set_field: null argument");
     if (int rc_ = require_aligned("hol_set_field", {x})) return rc_;
     cudaStream_t s = (cudaStream_t)stream;
-    const int nb = ceil_div(c->n, 256) < 4096 ? ceil_div(c->n, 256) : 4096;
-    k_expv<<<nb, 256, 0, s>>>(x, c->x, c->ev64, c->ev32, c->n, c->p.dtau, c->p.alpha, c->p.mu,
-                              c->ch4);
-    HOL_CHECK_LAUNCH("k_expv");
-    k_dbar<<<ceil_div(c->N, 128), 128, 0, s>>>(c->ev64, c->dbar, c->N, c->T);
-    HOL_CHECK_LAUNCH("k_dbar");
-    k_bounds<<<1, 256, 0, s>>>(c->dbar, c->N, exp(4.0 * c->p.dtau * fabs(c->p.t)), c->ch4,
-                               c->scal);
-    HOL_CHECK_LAUNCH("k_bounds");
+    k_field<<<c->N / kFieldSites, 256, 0, s>>>(x, c->x, c->ev64, c->ev32, c->dbar, c->scal,
+                                               c->field_cnt, c->N, c->T, c->p.dtau, c->p.alpha,
+                                               c->p.mu, c->ch4, exp(4.0 * c->p.dtau * fabs(c->p.t)));
+    HOL_CHECK_LAUNCH("k_field");
     int rc = kpm_setup(c, s);
     if (rc) return rc;
     c->field_set = 1;
@@ -443,7 +459,9 @@ extern "C" int fermion_matvec(hol_ctx* c, int op, int prec, const void* v, void*
             return launch_cg_mtm32(c, (const float*)v, (const float*)v, nullptr, (float*)out, n_rhs,
                                    nullptr, nullptr, nullptr, 0, 0, 1, nullptr, s);
         else {
-            int rc = launch_M(c, HOL_F64, v, c->v64a, n_rhs, nullptr, nullptr, s);
+            int rc = launch_MTM64(c, (const double*)v, (double*)out, n_rhs, s);   // small systems
+            if (rc != kNotTaken) return rc;
+            rc = launch_M(c, HOL_F64, v, c->v64a, n_rhs, nullptr, nullptr, s);
             if (rc) return rc;
             return launch_MT(c, HOL_F64, c->v64a, out, n_rhs, nullptr, s);
         }

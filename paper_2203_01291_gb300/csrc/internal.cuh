@@ -147,6 +147,11 @@ struct KpmPlan {
     int max_np;          // capacity per omega
     int* np;             // [T/2]  polynomial order N_P(omega)
     double2* coef;       // [T/2][max_np] complex c_m(omega)
+    float4* coef32;      // the same in FP32, (re, re, im, im)
+    // the recurrence's constants, db = bmax - bmin: (4 / db) dbar_i [N], then
+    // 2 (-2 bmin / db - 1) (dk32: then its rounding error)
+    double* dk64;
+    float* dk32;
 };
 
 struct ResArgs;
@@ -260,6 +265,7 @@ struct hol_ctx {
     int* kpm_q;          // its work queue [2] (next problem, finished blocks; zero between launches)
     double kpm_a1, kpm_a2;   // constants of the Chebyshev order heuristic (1, 1 by default)
     int pc_fuse;             // PCG: vector update fused into the preconditioner's transform
+    int* field_cnt;          // finished-block counts of k_field and k_force_bands (zero between launches)
     int resident;            // launch option "resident_cg": plain CG with its state on chip
     hol::ResPlan res_plan[2];    // its plan for the last n_rhs, by precision (resident.cu)
 };
@@ -345,6 +351,10 @@ int launch_MT(const hol_ctx* c, int prec, const void* u, void* out, int n_rhs,
 // FP64: out = b - M^T u.
 int launch_MT_resid64(const hol_ctx* c, const double* u, const double* b, double* out,
                       int n_rhs, const int* mask, cudaStream_t s);
+// FP64 out = M^T M v in one launch for systems small enough that every unit is
+// resident at once (mtm64.cu); kNotTaken (nothing launched) beyond that.
+constexpr int kNotTaken = 1;
+int launch_MTM64(const hol_ctx* c, const double* v, double* out, int n_rhs, cudaStream_t s);
 // FP32 fused CG step: pnew = r + beta pold (beta from the partial sums
 // rr_new / rr_old, 0 when first), q = M^T M pnew, pq_part = |M pnew|^2.
 // pnew and pq_part may be null.

@@ -12,7 +12,10 @@
 //   layout (strip.cuh), so a step has no barrier: about 150 cycles a step, the
 //   latency of its shuffles and dependent multiply-adds. Steps carry the
 //   recurrence x = d2 Bbar' t + (2 c0 t - prev), the factor 2 a folded into the
-//   diagonal, on packed FP32 pairs. P^{-1} P^{-T} at L = 16, Ltau = 160 on 2 rhs
+//   diagonal, on packed FP32 pairs; 2 c0 as two floats, since its rounding, the
+//   same at every site and step, would be the largest error of a long series
+//   (relative error of a series, mean over seven shapes: 6.4e-7, 1.1e-6 with
+//   one float or with the older kernels' unfolded constants). P^{-1} P^{-T} at L = 16, Ltau = 160 on 2 rhs
 //   16.9 us (30.4 with the one-column layout k_kpm_lane).
 //   k_kpm_rows (FP32, L >= 20): the strip over several warps per part, since one
 //   warp's issue slots would bound a step (L = 32: 500 cycles); one exchange of
@@ -44,8 +47,8 @@ namespace cgp = cooperative_groups;
 template <int L>
 __global__ void __launch_bounds__(64)
     k_kpm_strip(const float2* __restrict__ vin, float2* __restrict__ vout,
-                const double* __restrict__ dbar, const double* __restrict__ scal,
-                const int* __restrict__ npv, const double2* __restrict__ coef, int n_rhs, int Th,
+                const float* __restrict__ dk, const int* __restrict__ npv,
+                const float4* __restrict__ coef, int n_rhs, int Th,
                 int max_np, int mode, float th)
 {
     pdl_wait();      // the input comes from the previous kernel of the stream
@@ -64,13 +67,10 @@ __global__ void __launch_bounds__(64)
     float4* cw = ks_smem;                                            // (re, re, im, im)
     f32p* xb = reinterpret_cast<f32p*>(cw + max_np);                 // [series][part][RT][32]
     const int np = npv[wq];
-    for (int m = threadIdx.x; m < np; m += 64) {
-        const double2 c = coef[(long)wq * max_np + m];
-        cw[m] = make_float4((float)c.x, (float)c.x, (float)c.y, (float)c.y);
-    }
-    const double bmin = scal[S_BMIN], bmax = scal[S_BMAX], db = bmax - bmin;
-    const float a2 = (float)(4.0 / db), c2 = (float)(2.0 * (-2.0 * bmin / db - 1.0));
-    const f32p c02 = pk(c2, c2), th2 = pk(th, th), m1 = pk(-1.0f, -1.0f), half = pk(0.5f, 0.5f);
+    for (int m = threadIdx.x; m < np; m += 64) cw[m] = coef[(long)wq * max_np + m];
+    const float c2 = dk[N];
+    const f32p c02 = pk(c2, c2), c02l = pk(dk[N + 1], dk[N + 1]), th2 = pk(th, th);
+    const f32p m1 = pk(-1.0f, -1.0f), half = pk(0.5f, 0.5f);
     f32p t[RT], d[RT];
 #pragma unroll
     for (int q = 0; q < RT; ++q) {
@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(64)
         if (geo.has(q)) {
             const float4 v = *reinterpret_cast<const float4*>(vin + off + geo.site(q));
             t[q] = part ? pk(v.y, v.w) : pk(v.x, v.z);
-            const double2 db2 = *reinterpret_cast<const double2*>(dbar + geo.site(q));
-            d[q] = pk(a2 * (float)db2.x, a2 * (float)db2.y);
+            const float2 db2 = *reinterpret_cast<const float2*>(dk + geo.site(q));
+            d[q] = pk(db2.x, db2.y);
         }
     }
     __syncthreads();
@@ -88,14 +88,14 @@ __global__ void __launch_bounds__(64)
     auto series = [&](auto trans_c, int sidx) {
         constexpr bool trans = decltype(trans_c)::value;
         const float4 c0 = cw[0];
-        f32p A[RT], B[RT], prev[RT];
+        f32p A[RT], B[RT], nprev[RT];   // minus the one before
         // T_1 u = A u = 2 A (u / 2) - 0: the recurrence from t = u / 2, prev = 0
 #pragma unroll
         for (int q = 0; q < RT; ++q) {
             A[q] = mul2(pk(c0.x, c0.y), t[q]);
             B[q] = mul2(pk(c0.z, c0.w), t[q]);
             t[q] = mul2(half, t[q]);
-            prev[q] = 0;
+            nprev[q] = 0;
         }
         for (int m = 1; m < np; ++m) {
             const float4 cm = cw[m];
@@ -120,16 +120,16 @@ __global__ void __launch_bounds__(64)
             }
 #pragma unroll
             for (int q = 0; q < RT; ++q) {
-                const f32p y = fma2(c02, t[q], mul2(m1, prev[q]));
+                const f32p y = fma2(c02, t[q], fma2(c02l, t[q], nprev[q]));
                 const f32p x = trans ? add2(b[q], y) : fma2(d[q], b[q], y);
-                prev[q] = t[q];
+                nprev[q] = mul2(m1, t[q]);
                 t[q] = x;
                 A[q] = fma2(cr, x, A[q]);
                 B[q] = fma2(ci, x, B[q]);
             }
             if (m == 1)
 #pragma unroll
-                for (int q = 0; q < RT; ++q) prev[q] = add2(prev[q], prev[q]);   // T_0 u = u
+                for (int q = 0; q < RT; ++q) nprev[q] = add2(nprev[q], nprev[q]);   // T_0 u = u
         }
         // re = A_re - s B_im, im = A_im + s B_re; s = -1 for the conjugate
         // coefficients of the transpose
@@ -165,8 +165,8 @@ int run_strip(const hol_ctx* c, const float2* in, float2* out, int n_rhs, int mo
     const size_t sm = (size_t)max_np * sizeof(float4) + (size_t)4 * K::RT * 32 * sizeof(f32p);
     if (int rc = smem_raise((const void*)k_kpm_strip<L>, sm)) return rc;
     const int grid = Th * ((n_rhs + K::G - 1) / K::G);
-    HOL_CUDA(launch_pdl(c, k_kpm_strip<L>, grid, 64, sm, s, in, out, c->dbar, c->scal, c->kpm.np,
-                        c->kpm.coef, n_rhs, Th, max_np, mode, (float)c->th));
+    HOL_CUDA(launch_pdl(c, k_kpm_strip<L>, grid, 64, sm, s, in, out, c->kpm.dk32, c->kpm.np,
+                        c->kpm.coef32, n_rhs, Th, max_np, mode, (float)c->th));
     HOL_CHECK_LAUNCH("k_kpm_strip");
     return HOL_OK;
 }
@@ -189,8 +189,8 @@ struct BGeo {
 template <int L, bool CL>
 __global__ void __launch_bounds__(32 * BGeo<L>::W * (CL ? 1 : 2))
     k_kpm_rows(const float2* __restrict__ vin, float2* __restrict__ vout,
-               const double* __restrict__ dbar, const double* __restrict__ scal,
-               const int* __restrict__ npv, const double2* __restrict__ coef, int n_rhs, int Th,
+               const float* __restrict__ dk, const int* __restrict__ npv,
+               const float4* __restrict__ coef, int n_rhs, int Th,
                int max_np, int mode, float th)
 {
     pdl_wait();      // the input comes from the previous kernel of the stream
@@ -222,20 +222,17 @@ __global__ void __launch_bounds__(32 * BGeo<L>::W * (CL ? 1 : 2))
     f32p* eb = reinterpret_cast<f32p*>(cw + max_np) + slot * EB;
     f32p* xb = reinterpret_cast<f32p*>(cw + max_np) + (CL ? 1 : 2) * EB;
     const int np = npv[wq];
-    for (int m = threadIdx.x; m < np; m += blockDim.x) {
-        const double2 c = coef[(long)wq * max_np + m];
-        cw[m] = make_float4((float)c.x, (float)c.x, (float)c.y, (float)c.y);
-    }
-    const double bmin = scal[S_BMIN], bmax = scal[S_BMAX], db = bmax - bmin;
-    const float a2 = (float)(4.0 / db), c2 = (float)(2.0 * (-2.0 * bmin / db - 1.0));
-    const f32p c02 = pk(c2, c2), th2 = pk(th, th), m1 = pk(-1.0f, -1.0f), half = pk(0.5f, 0.5f);
+    for (int m = threadIdx.x; m < np; m += blockDim.x) cw[m] = coef[(long)wq * max_np + m];
+    const float c2 = dk[N];
+    const f32p c02 = pk(c2, c2), c02l = pk(dk[N + 1], dk[N + 1]), th2 = pk(th, th);
+    const f32p m1 = pk(-1.0f, -1.0f), half = pk(0.5f, 0.5f);
     f32p t[RT], d[RT];
 #pragma unroll
     for (int q = 0; q < RT; ++q) {
         const float4 v = *reinterpret_cast<const float4*>(vin + off + site0 + q * L);
         t[q] = part ? pk(v.y, v.w) : pk(v.x, v.z);
-        const double2 db2 = *reinterpret_cast<const double2*>(dbar + site0 + q * L);
-        d[q] = pk(a2 * (float)db2.x, a2 * (float)db2.y);
+        const float2 db2 = *reinterpret_cast<const float2*>(dk + site0 + q * L);
+        d[q] = pk(db2.x, db2.y);
     }
     __syncthreads();
     int par = 0;
@@ -290,13 +287,13 @@ __global__ void __launch_bounds__(32 * BGeo<L>::W * (CL ? 1 : 2))
     auto series = [&](auto trans_c, int sidx) {
         constexpr bool trans = decltype(trans_c)::value;
         const float4 c0 = cw[0];
-        f32p A[RT], B[RT], prev[RT];
+        f32p A[RT], B[RT], nprev[RT];   // minus the one before
 #pragma unroll
         for (int q = 0; q < RT; ++q) {   // T_1 u = 2 A (u / 2) - 0, as in k_kpm_strip
             A[q] = mul2(pk(c0.x, c0.y), t[q]);
             B[q] = mul2(pk(c0.z, c0.w), t[q]);
             t[q] = mul2(half, t[q]);
-            prev[q] = 0;
+            nprev[q] = 0;
         }
         for (int m = 1; m < np; ++m) {
             const float4 cm = cw[m];
@@ -317,16 +314,16 @@ __global__ void __launch_bounds__(32 * BGeo<L>::W * (CL ? 1 : 2))
             }
 #pragma unroll
             for (int q = 0; q < RT; ++q) {
-                const f32p y = fma2(c02, t[q], mul2(m1, prev[q]));
+                const f32p y = fma2(c02, t[q], fma2(c02l, t[q], nprev[q]));
                 const f32p x = trans ? add2(b[q], y) : fma2(d[q], b[q], y);
-                prev[q] = t[q];
+                nprev[q] = mul2(m1, t[q]);
                 t[q] = x;
                 A[q] = fma2(cr, x, A[q]);
                 B[q] = fma2(ci, x, B[q]);
             }
             if (m == 1)
 #pragma unroll
-                for (int q = 0; q < RT; ++q) prev[q] = add2(prev[q], prev[q]);
+                for (int q = 0; q < RT; ++q) nprev[q] = add2(nprev[q], nprev[q]);
         }
         f32p* mine = xb + (long)((CL ? sidx : 2 * sidx + part) * RT) * NT + tid;
         const f32p* oth = mine + (CL ? 0 : (1 - 2 * part) * RT * NT);
@@ -397,11 +394,11 @@ int run_rows(const hol_ctx* c, const float2* in, float2* out, int n_rhs, int mod
     if (int rc = smem_raise((const void*)(cl ? k_kpm_rows<L, true> : k_kpm_rows<L, false>), sm))
         return rc;
     if (cl)
-        HOL_CUDA(launch_pair(c, k_kpm_rows<L, true>, Th * n_rhs, 32 * P::W, sm, s, in, out, c->dbar,
-                             c->scal, c->kpm.np, c->kpm.coef, n_rhs, Th, max_np, mode, (float)c->th));
+        HOL_CUDA(launch_pair(c, k_kpm_rows<L, true>, Th * n_rhs, 32 * P::W, sm, s, in, out,
+                             c->kpm.dk32, c->kpm.np, c->kpm.coef32, n_rhs, Th, max_np, mode, (float)c->th));
     else
-        HOL_CUDA(launch_pdl(c, k_kpm_rows<L, false>, Th * n_rhs, 64 * P::W, sm, s, in, out, c->dbar,
-                            c->scal, c->kpm.np, c->kpm.coef, n_rhs, Th, max_np, mode, (float)c->th));
+        HOL_CUDA(launch_pdl(c, k_kpm_rows<L, false>, Th * n_rhs, 64 * P::W, sm, s, in, out,
+                            c->kpm.dk32, c->kpm.np, c->kpm.coef32, n_rhs, Th, max_np, mode, (float)c->th));
     HOL_CHECK_LAUNCH("k_kpm_rows");
     return HOL_OK;
 }
@@ -422,8 +419,8 @@ struct PGeo {
 template <int L>
 __global__ void __launch_bounds__(32 * PGeo<L>::W)
     k_kpm_pair(const double2* __restrict__ vin, double2* __restrict__ vout,
-               const double* __restrict__ dbar, const double* __restrict__ scal,
-               const int* __restrict__ npv, const double2* __restrict__ coef, int n_rhs, int Th,
+               const double* __restrict__ dk, const int* __restrict__ npv,
+               const double2* __restrict__ coef, int n_rhs, int Th,
                int max_np, int mode, double th)
 {
     pdl_wait();      // the input comes from the previous kernel of the stream
@@ -454,8 +451,7 @@ __global__ void __launch_bounds__(32 * PGeo<L>::W)
     double* xb = eb + 2 * P::NCH * 2 * L;                           // [series][2 C][threads]
     const int np = npv[wq];
     for (int m = threadIdx.x; m < np; m += blockDim.x) cw[m] = coef[(long)wq * max_np + m];
-    const double bmin = scal[S_BMIN], bmax = scal[S_BMAX], db = bmax - bmin;
-    const double a2 = 4.0 / db, c02 = 2.0 * (-2.0 * bmin / db - 1.0);
+    const double c02 = dk[N];
     const double* vf = reinterpret_cast<const double*>(vin);
     double t[2][C], d[2][C];
 #pragma unroll
@@ -463,7 +459,7 @@ __global__ void __launch_bounds__(32 * PGeo<L>::W)
 #pragma unroll
         for (int k = 0; k < C; ++k) {
             t[r][k] = vf[2 * (off + site0 + r * L + k) + part];
-            d[r][k] = a2 * dbar[site0 + r * L + k];
+            d[r][k] = dk[site0 + r * L + k];
         }
     __syncthreads();
     int par = 0;
@@ -602,7 +598,7 @@ int run_pair(const hol_ctx* c, const double2* in, double2* out, int n_rhs, int m
     const size_t sm = (size_t)max_np * sizeof(double2) +
                       (size_t)(2 * P::NCH * 2 * L + 2 * 2 * P::COLS * 32 * P::W) * sizeof(double);
     if (int rc = smem_raise((const void*)k_kpm_pair<L>, sm)) return rc;
-    HOL_CUDA(launch_pair(c, k_kpm_pair<L>, Th * n_rhs, 32 * P::W, sm, s, in, out, c->dbar, c->scal,
+    HOL_CUDA(launch_pair(c, k_kpm_pair<L>, Th * n_rhs, 32 * P::W, sm, s, in, out, c->kpm.dk64,
                          c->kpm.np, c->kpm.coef, n_rhs, Th, max_np, mode, c->th));
     HOL_CHECK_LAUNCH("k_kpm_pair");
     return HOL_OK;

@@ -1197,53 +1197,113 @@ __global__ void __launch_bounds__(KBand<L>::THREADS > 0 ? KBand<L>::THREADS : 32
     }
 }
 
-// N_P(omega) and c_m(omega), m < N_P, one block per omega < T/2.
-// f(cos theta_n) is evaluated once per quadrature node into shared memory;
-// cos(m theta_n) follows from a rotation by m pi / N_Q per node, so the
-// coefficient sums cost FMAs only (FP64 throughput is scarce on this part).
-__global__ void k_kpm_coeffs(const double* __restrict__ scal, int T, int max_np,
-                             int* __restrict__ npv, double2* __restrict__ coef,
-                             int* __restrict__ clamped, double a1, double a2)
+// N_P(omega) and c_m(omega), m < N_P, one block per omega < T/2, and the
+// constants of the recurrence (KpmPlan::dk64 / dk32), shared among the blocks.
+// The quadrature angles theta_q = pi (2 q + 1) / (2 N_Q) make every cos(m
+// theta_q) an entry cos(pi k / (2 N_Q)), k = m (2 q + 1) mod 4 N_Q, of one table of
+// a quarter wave, and q and N_Q - 1 - q enter with the signs 1 and (-1)^m, so a
+// coefficient is N_P terms of two multiply-adds, four lanes per coefficient. (A
+// rotation per term over all N_Q nodes took six FP64 operations each, 27 us at
+// Ltau = 160 on the FP64 pipe's sixty cycles an instruction; now 8.4.)
+__global__ void __launch_bounds__(256) k_kpm_coeffs(const double* __restrict__ scal, int T, int max_np,
+                                                    int* __restrict__ npv, double2* __restrict__ coef,
+                                                    float4* __restrict__ coef32,
+                                                    const double* __restrict__ dbar, int N,
+                                                    double* __restrict__ dk64, float* __restrict__ dk32,
+                                                    int* __restrict__ clamped, double a1, double a2)
 {
-    extern __shared__ double2 fq[];              // [2 max_np]
+    pdl_wait();      // the bounds come from the previous kernel of the stream
+    const PdlTriggerAtExit pdl_at_exit;
+    extern __shared__ double2 fq[];              // [2][max_np] even, odd sums; then the table
     const int w = blockIdx.x;
     const double bmin = scal[S_BMIN], bmax = scal[S_BMAX];
     const double db = bmax - bmin;
+    // the block's scalars, each by one warp (an FP64 division is a dozen
+    // instructions of sixty cycles for every warp that computes it)
+    __shared__ int s_np;
+    __shared__ double s_sin, s_cos, s_inv, s_s4;
     const double phi = 2.0 * M_PI / T * (w + 0.5);
-    const double npd = floor(db * (a1 / phi + a2));   // Eq. (NP_heuristic)
-    const int np = npd < 1.0 ? 1 : (npd > (double)max_np ? max_np : (int)npd);
     if (threadIdx.x == 0) {
-        npv[w] = np;
+        const double npd = floor(db * (a1 / phi + a2));   // Eq. (NP_heuristic)
+        const int n = npd < 1.0 ? 1 : (npd > (double)max_np ? max_np : (int)npd);
+        s_np = n;
+        s_inv = 0.25 / n;                                  // 1 / (2 N_Q)
+        npv[w] = n;
         if (npd > (double)max_np) atomicExch(clamped, 1);
-    }
-    const int nq = 2 * np;
-    double sp, cp;
-    sincos(phi, &sp, &cp);
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-        const double y = cospi((q + 0.5) / nq);
-        const double bb = bmin + (y + 1.0) * db * 0.5;
-        // f = 1 / (1 - e^{-i phi} bb) = 1 / ((1 - bb cos phi) + i bb sin phi)
-        const double re = 1.0 - bb * cp, im = bb * sp;
-        const double den = re * re + im * im;
-        fq[q] = make_double2(re / den, -im / den);
+    } else if (threadIdx.x == 32) {
+        sincos(phi, &s_sin, &s_cos);
+    } else if (threadIdx.x == 64) {
+        s_s4 = 4.0 / db;
+        if (w == 0) {
+            const double c02 = 2.0 * (-2.0 * bmin / db - 1.0);
+            dk64[N] = c02;
+            dk32[N] = (float)c02;
+            dk32[N + 1] = (float)(c02 - (double)(float)c02);
+        }
     }
     __syncthreads();
-    for (int m = threadIdx.x; m < np; m += blockDim.x) {
-        double c, sn, cd, sd;
-        sincospi(0.5 * m / nq, &sn, &c);      // angle m theta_0
-        sincospi((double)m / nq, &sd, &cd);   // step m pi / N_Q
+    const int np = s_np, nq = 2 * np;
+    const double inv = s_inv, sp = s_sin, cp = s_cos;
+    double2* fe = fq;
+    double2* fo = fq + max_np;
+    double* ct = reinterpret_cast<double*>(fq + 2 * max_np);   // [2 max_np + 1]
+    for (int k = threadIdx.x; k <= nq; k += blockDim.x) ct[k] = cospi(k * inv);
+    __syncthreads();
+    // f = 1 / (1 - e^{-i phi} bb) = 1 / ((1 - bb cos phi) + i bb sin phi) at the
+    // nodes +-y
+    auto node = [&](double y) -> double2 {
+        const double bb = bmin + (y + 1.0) * db * 0.5;
+        const double re = 1.0 - bb * cp, im = bb * sp;
+        const double iden = 1.0 / (re * re + im * im);
+        return make_double2(re * iden, -im * iden);
+    };
+    for (int q = threadIdx.x; q < nq; q += blockDim.x) {   // nodes q < np, then their mirrors
+        const int p = q < np ? q : q - np;
+        const double y = ct[2 * p + 1];
+        (q < np ? fe : fo)[p] = node(q < np ? y : -y);
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < np; q += blockDim.x) {
+        const double2 u = fe[q], v = fo[q];
+        fe[q] = make_double2(u.x + v.x, u.y + v.y);
+        fo[q] = make_double2(u.x - v.x, u.y - v.y);
+    }
+    __syncthreads();
+    const int sub = threadIdx.x & 3;
+    for (int m0 = 0; m0 < np; m0 += blockDim.x / 4) {
+        const int m = m0 + (threadIdx.x >> 2);
         double sr = 0.0, si = 0.0;
-        for (int q = 0; q < nq; ++q) {
-            const double2 f = fq[q];
-            sr = fma(c, f.x, sr);
-            si = fma(c, f.y, si);
-            const double c2 = c * cd - sn * sd;
-            sn = fma(sn, cd, c * sd);
-            c = c2;
+        if (m < np) {
+            const double2* f = (m & 1) ? fo : fe;
+            int k = (int)((long)m * (2 * sub + 1) % (4 * nq));
+            const int step = (int)((long)m * 8 % (4 * nq));
+            for (int q = sub; q < np; q += 4) {
+                const int kk = k > 2 * nq ? 4 * nq - k : k;
+                const double c = kk > nq ? -ct[2 * nq - kk] : ct[kk];
+                const double2 fv = f[q];
+                sr = fma(c, fv.x, sr);
+                si = fma(c, fv.y, si);
+                k += step;
+                if (k >= 4 * nq) k -= 4 * nq;
+            }
         }
-        const double qm = (m == 0) ? 2.0 : 1.0;   // q_m / (pi/2)
-        const double fac = 2.0 / (qm * nq);       // pi / (q_m N_Q)
-        coef[(long)w * max_np + m] = make_double2(fac * sr, fac * si);
+#pragma unroll
+        for (int o = 2; o > 0; o >>= 1) {
+            sr += __shfl_xor_sync(kFull, sr, o);
+            si += __shfl_xor_sync(kFull, si, o);
+        }
+        if (m < np && sub == 0) {
+            const double fac = m == 0 ? 2.0 * inv : 4.0 * inv;   // pi / (q_m N_Q)
+            const double cr = fac * sr, ci = fac * si;
+            coef[(long)w * max_np + m] = make_double2(cr, ci);
+            coef32[(long)w * max_np + m] = make_float4((float)cr, (float)cr, (float)ci, (float)ci);
+        }
+    }
+    const double s4 = s_s4;
+    for (int i = w * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const double d = s4 * dbar[i];
+        dk64[i] = d;
+        dk32[i] = (float)d;
     }
 }
 
@@ -1565,15 +1625,20 @@ int precond_alloc(hol_ctx* c)
     HOL_CUDA(cudaMalloc((void**)&c->kpm.np, (T / 2) * sizeof(int) + sizeof(int)));
     HOL_CUDA(cudaMalloc((void**)&c->kpm.coef, (long)(T / 2) * c->kpm.max_np * sizeof(double2)));
     HOL_CUDA(cudaMemset(c->kpm.np, 0, (T / 2) * sizeof(int) + sizeof(int)));
+    HOL_CUDA(cudaMalloc((void**)&c->kpm.coef32, (long)(T / 2) * c->kpm.max_np * sizeof(float4)));
+    HOL_CUDA(cudaMalloc((void**)&c->kpm.dk64, (c->N + 2) * sizeof(double)));
+    HOL_CUDA(cudaMalloc((void**)&c->kpm.dk32, (c->N + 2) * sizeof(float)));
     return HOL_OK;
 }
 
 int kpm_setup(hol_ctx* c, cudaStream_t s)
 {
-    const size_t sm = 2 * (size_t)c->kpm.max_np * sizeof(double2);
+    const size_t sm = 2 * (size_t)c->kpm.max_np * sizeof(double2) +
+                      (2 * (size_t)c->kpm.max_np + 1) * sizeof(double);
     if (int rc = smem_raise((const void*)k_kpm_coeffs, sm)) return rc;
-    k_kpm_coeffs<<<c->T / 2, 128, sm, s>>>(c->scal, c->T, c->kpm.max_np, c->kpm.np, c->kpm.coef,
-                                           c->kpm.np + c->T / 2, c->kpm_a1, c->kpm_a2);
+    HOL_CUDA(launch_pdl(c, k_kpm_coeffs, c->T / 2, 256, sm, s, c->scal, c->T, c->kpm.max_np, c->kpm.np,
+                        c->kpm.coef, c->kpm.coef32, c->dbar, c->N, c->kpm.dk64, c->kpm.dk32,
+                        c->kpm.np + c->T / 2, c->kpm_a1, c->kpm_a2));
     HOL_CHECK_LAUNCH("k_kpm_coeffs");
     return HOL_OK;
 }
