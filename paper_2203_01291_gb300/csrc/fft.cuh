@@ -90,6 +90,19 @@ __device__ __forceinline__ void dft_small(typename Cx<R>::T2 (&a)[RAD],
         a[1] = cadd(d02, d13);
         a[2] = csub(s02, s13);
         a[3] = csub(d02, d13);
+    } else if constexpr (RAD == 8) {   // two of length 4, the odd one turned by root^q
+        C2 e[4] = {a[0], a[2], a[4], a[6]}, o[4] = {a[1], a[3], a[5], a[7]};
+        const C2 r4[4] = {root[0], root[2], root[4], root[6]};
+        dft_small<R, 4>(e, r4);
+        dft_small<R, 4>(o, r4);
+        o[1] = cmul(o[1], root[1]);
+        o[2] = cmi(o[2]);
+        o[3] = cmul(o[3], root[3]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            a[q] = cadd(e[q], o[q]);
+            a[q + 4] = csub(e[q], o[q]);
+        }
     } else {
         constexpr int HF = (RAD - 1) / 2;
         C2 s[HF], d[HF];
@@ -200,17 +213,26 @@ __device__ typename Cx<R>::T2* fft_tau(typename Cx<R>::T2* a, typename Cx<R>::T2
 // The same transform with the length T, the tile width TS and the block size
 // NT known at compile time (the lengths of the configured workloads): the
 // plan, the butterfly loops and every index division are resolved by the
-// compiler. Same passes and twiddles as fft_tau.
+// compiler. Twiddles as in fft_tau, from shared memory.
 // ---------------------------------------------------------------------------
 struct PlanCT {
     int n;
     int r[16];
 };
 
-__host__ __device__ constexpr PlanCT plan_ct(int T)
+// FP32: an odd power of two from 8 on takes one radix 8 pass in place of a 4 and
+// a 2 (a pass costs a barrier and a trip through shared memory, some 200
+// cycles). FP64 passes are bound by the FP64 pipe and spread over more warps
+// with the smaller radices.
+__host__ __device__ constexpr PlanCT plan_ct(int T, bool fp32)
 {
     PlanCT p{0, {}};
-    int t = T;
+    int t = T, e2 = 0;
+    for (int u = T; u % 2 == 0; u /= 2) ++e2;
+    if (fp32 && e2 >= 3 && e2 % 2 == 1) {
+        p.r[p.n++] = 8;
+        t /= 8;
+    }
     const int rs[5] = {4, 2, 3, 5, 7};
     for (int k = 0; k < 5; ++k)
         while (t % rs[k] == 0 && p.n < 16) {
@@ -260,7 +282,7 @@ __device__ __forceinline__ typename Cx<R>::T2* fft_tau_ct(typename Cx<R>::T2* a,
                                                           typename Cx<R>::T2* b,
                                                           const typename Cx<R>::T2* __restrict__ w2)
 {
-    constexpr PlanCT P = plan_ct(T);
+    constexpr PlanCT P = plan_ct(T, sizeof(R) == 4);
     static_assert(P.n > 0, "length with a prime factor above 7");
     if constexpr (S < P.n) {
         constexpr int RAD = P.r[S];

@@ -15,8 +15,9 @@
 //   diagonal, on packed FP32 pairs; 2 c0 as two floats, since its rounding, the
 //   same at every site and step, would be the largest error of a long series
 //   (relative error of a series, mean over seven shapes: 6.4e-7, 1.1e-6 with
-//   one float or with the older kernels' unfolded constants). P^{-1} P^{-T} at L = 16, Ltau = 160 on 2 rhs
-//   16.9 us (30.4 with the one-column layout k_kpm_lane).
+//   one float or with the older kernels' unfolded constants). P^{-1} P^{-T} at
+//   L = 16, Ltau = 160 on 2 rhs 15.2 us (30.4 with the one-column layout
+//   k_kpm_lane); 13.8 with the set-up ahead of the wait for the forward transform.
 //   k_kpm_rows (FP32, L >= 20): the strip over several warps per part, since one
 //   warp's issue slots would bound a step (L = 32: 500 cycles); one exchange of
 //   edge rows per step. L = 32, Ltau = 200: 24.7 us on 2 rhs (41.0 with k_kpm_reg).
@@ -51,8 +52,6 @@ __global__ void __launch_bounds__(64)
                 const float4* __restrict__ coef, int n_rhs, int Th,
                 int max_np, int mode, float th)
 {
-    pdl_wait();      // the input comes from the previous kernel of the stream
-    const PdlTriggerAtExit pdl_at_exit;
     using K = RGeo<L>;
     constexpr int N = L * L, RT = K::RT;
     const K geo;
@@ -74,13 +73,20 @@ __global__ void __launch_bounds__(64)
     f32p t[RT], d[RT];
 #pragma unroll
     for (int q = 0; q < RT; ++q) {
-        t[q] = 0;
         d[q] = 0;
+        if (geo.has(q)) {
+            const float2 db2 = *reinterpret_cast<const float2*>(dk + geo.site(q));
+            d[q] = pk(db2.x, db2.y);
+        }
+    }
+    pdl_wait();      // the input comes from the previous kernel of the stream
+    pdl_trigger();   // the next kernel's blocks may take their places (it waits for this one's end)
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+        t[q] = 0;
         if (geo.has(q)) {
             const float4 v = *reinterpret_cast<const float4*>(vin + off + geo.site(q));
             t[q] = part ? pk(v.y, v.w) : pk(v.x, v.z);
-            const float2 db2 = *reinterpret_cast<const float2*>(dk + geo.site(q));
-            d[q] = pk(db2.x, db2.y);
         }
     }
     __syncthreads();
@@ -193,8 +199,6 @@ __global__ void __launch_bounds__(32 * BGeo<L>::W * (CL ? 1 : 2))
                const float4* __restrict__ coef, int n_rhs, int Th,
                int max_np, int mode, float th)
 {
-    pdl_wait();      // the input comes from the previous kernel of the stream
-    const PdlTriggerAtExit pdl_at_exit;
     using P = BGeo<L>;
     constexpr int N = L * L, LP = P::LP, RT = 2 * P::RP, NT = 32 * P::W;
     // CL: a cluster of two blocks, one per part; else both parts in one block
@@ -229,10 +233,15 @@ __global__ void __launch_bounds__(32 * BGeo<L>::W * (CL ? 1 : 2))
     f32p t[RT], d[RT];
 #pragma unroll
     for (int q = 0; q < RT; ++q) {
-        const float4 v = *reinterpret_cast<const float4*>(vin + off + site0 + q * L);
-        t[q] = part ? pk(v.y, v.w) : pk(v.x, v.z);
         const float2 db2 = *reinterpret_cast<const float2*>(dk + site0 + q * L);
         d[q] = pk(db2.x, db2.y);
+    }
+    pdl_wait();      // the input comes from the previous kernel of the stream
+    pdl_trigger();   // the next kernel's blocks may take their places (it waits for this one's end)
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(vin + off + site0 + q * L);
+        t[q] = part ? pk(v.y, v.w) : pk(v.x, v.z);
     }
     __syncthreads();
     int par = 0;
@@ -423,8 +432,6 @@ __global__ void __launch_bounds__(32 * PGeo<L>::W)
                const double2* __restrict__ coef, int n_rhs, int Th,
                int max_np, int mode, double th)
 {
-    pdl_wait();      // the input comes from the previous kernel of the stream
-    const PdlTriggerAtExit pdl_at_exit;
     using P = PGeo<L>;
     constexpr int N = L * L, C = P::COLS, LP = P::LP;
     const cgp::cluster_group cl = cgp::this_cluster();
@@ -457,10 +464,13 @@ __global__ void __launch_bounds__(32 * PGeo<L>::W)
 #pragma unroll
     for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int k = 0; k < C; ++k) {
-            t[r][k] = vf[2 * (off + site0 + r * L + k) + part];
-            d[r][k] = dk[site0 + r * L + k];
-        }
+        for (int k = 0; k < C; ++k) d[r][k] = dk[site0 + r * L + k];
+    pdl_wait();      // the input comes from the previous kernel of the stream
+    const PdlTriggerAtExit pdl_at_exit;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int k = 0; k < C; ++k) t[r][k] = vf[2 * (off + site0 + r * L + k) + part];
     __syncthreads();
     int par = 0;
     // odd y-bonds: this chunk's rows with its neighbours' (through shared memory)

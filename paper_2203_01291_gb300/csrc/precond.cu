@@ -96,6 +96,25 @@ __device__ __forceinline__ void st_cpair(double2* p, double2 a, double2 b)
     p[1] = b;
 }
 
+// Dependent-launch trigger of the transforms: at once in FP32, which hides the
+// next kernel's launch and set-up; at the end in FP64, where the next kernel's
+// blocks would be placed while these hold shared memory, so that two long FP64
+// series land on one multiprocessor and take twice as long (P^{-1} P^{-T},
+// L = 20, Ltau = 120, 2 rhs: 133 us at once, 121 at the end).
+//
+// What bounds the transforms in FP32 on few right-hand sides is latency: the
+// input, a barrier and a trip through shared memory per pass, the sums. So the
+// twiddles wait in shared memory, an odd power of two takes a radix 8 pass
+// (fft.cuh), and the joined update and the r.z sum stay off the FP64 pipe.
+// P^{-1} P^{-T}, L = 16, Ltau = 160, 2 rhs: 15.2 -> 13.8 us; L = 32, Ltau = 200,
+// 16 rhs: 48.4 -> 40; a preconditioned iteration at L = 16, Ltau = 160, 2 rhs, all
+// kernels: 27.6 -> 24.5 us.
+template <bool EARLY>
+struct PdlTriggerFp32 {
+    __device__ __forceinline__ PdlTriggerFp32() { if (EARLY) pdl_trigger(); }
+    __device__ __forceinline__ ~PdlTriggerFp32() { if (!EARLY) pdl_trigger(); }
+};
+
 // The tau transforms act on real site lines, two per complex transform: the
 // tile holds TS sites as TS / 2 columns, site 2c in the real and site 2c + 1
 // in the imaginary part of column c.
@@ -111,12 +130,21 @@ __device__ __forceinline__ void st_cpair(double2* p, double2 a, double2 b)
 template <typename R, int TC = 0, int TSC = 0>
 __global__ void __launch_bounds__(256) k_tau_fwd(const R* __restrict__ v,
                                                  typename Cx<R>::T2* __restrict__ vh,
-                                                 const typename Cx<R>::T2* __restrict__ w2, int T_,
+                                                 const typename Cx<R>::T2* __restrict__ w2g, int T_,
                                                  int N, int TS_, RadixPlan plan, R scale)
 {
-    pdl_wait();      // the input comes from the previous kernel of the stream
-    const PdlTriggerAtExit pdl_at_exit;
     using C2 = typename Cx<R>::T2;
+    // the twiddles come to shared memory while the previous kernel ends (read
+    // from L2 in every pass they cost each its latency)
+    const C2* w2 = w2g;
+    if constexpr (TC > 0) {
+        __shared__ C2 tws[2 * TC];
+        for (int k = threadIdx.x; k < 2 * TC; k += 256) tws[k] = w2g[k];
+        w2 = tws;
+    }
+    pdl_wait();      // the input comes from the previous kernel of the stream
+    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
+    __syncthreads();
     const int T = TC > 0 ? TC : T_;
     const int TS = TSC > 0 ? TSC : TS_;
     const int TH = TS / 2;                 // transform columns
@@ -180,13 +208,26 @@ struct PcUpdK {
 template <typename R, int TC = 0, int TSC = 0>
 __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
                                                      typename Cx<R>::T2* __restrict__ vh,
-                                                     const typename Cx<R>::T2* __restrict__ w2,
+                                                     const typename Cx<R>::T2* __restrict__ w2g,
                                                      int T_, int N, int TS_, RadixPlan plan,
                                                      R scale, PcUpdK<R> u)
 {
-    pdl_wait();      // p, q and the partials come from the previous kernel of the stream
-    const PdlTriggerAtExit pdl_at_exit;
     using C2 = typename Cx<R>::T2;
+    // The first kUpdItems elements of a thread (FP32: all of them at the configured
+    // lengths) are loaded before alpha is formed, a chain of partial sums and an
+    // FP64 division that would otherwise precede the loads' latency. In FP64 more
+    // than one costs registers and gains nothing.
+    constexpr int kUpdItems = sizeof(R) == 4 ? 4 : 1;
+    // the twiddles come to shared memory while the previous kernel ends (read
+    // from L2 in every pass they cost each its latency)
+    const C2* w2 = w2g;
+    if constexpr (TC > 0) {
+        __shared__ C2 tws[2 * TC];
+        for (int k = threadIdx.x; k < 2 * TC; k += 256) tws[k] = w2g[k];
+        w2 = tws;
+    }
+    pdl_wait();      // p, q and the partials come from the previous kernel of the stream
+    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
     const int T = TC > 0 ? TC : T_;
     const int TS = TSC > 0 ? TSC : TS_;
     const int TH = TS / 2;                 // transform columns
@@ -197,12 +238,43 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
     const int i0 = blockIdx.x * TS;
     const long base = (long)rhs * T * N;
     const bool act = u.mask == nullptr || u.mask[rhs] != 0;
+    struct Item {
+        R r[2], q[2], x[2], p[2], pp[2];
+    };
+    // element `item` of the tile: its memory offset, or -1 outside the lattice
+    auto offset = [&](int item) -> long {
+        const int c = item % TH, tau = item / TH, i = i0 + 2 * c;
+        return item < T * TH && i < N ? base + (long)tau * N + i : -1;   // N is even: i + 1 < N too
+    };
+    auto load = [&](long o, Item& e) {
+        e.r[0] = e.r[1] = R(0);
+        if (o < 0) return;
+        ld_pair(v + o, e.r[0], e.r[1]);
+        if (!act) return;
+        ld_pair(u.q + o, e.q[0], e.q[1]);
+        if (u.fold != 0) {
+            ld_pair(u.x + o, e.x[0], e.x[1]);
+            ld_pair(u.p + o, e.p[0], e.p[1]);
+            if (u.fold == 2) ld_pair(u.pp + o, e.pp[0], e.pp[1]);
+        }
+    };
+    Item pre[kUpdItems];
+#pragma unroll
+    for (int k = 0; k < kUpdItems; ++k) load(offset(threadIdx.x + k * 256), pre[k]);
     __shared__ double s_alpha, s_alpha_prev;
     if (threadIdx.x < 32) {
         double al = 0.0, alp = 0.0;
         if (act) {
-            const double pq = warp_sum_array(u.pq_part + (long)rhs * u.pq_stride, u.pq_n);
-            const double dz = warp_sum_array(u.dz_part + (long)rhs * kRedStride, u.dz_n);
+            // the two sums in the two halves of the warp
+            const int half = threadIdx.x >> 4, l16 = threadIdx.x & 15;
+            const double* src = half ? u.dz_part + (long)rhs * kRedStride
+                                     : u.pq_part + (long)rhs * u.pq_stride;
+            const int cnt = half ? u.dz_n : u.pq_n;
+            double t = 0.0;
+            for (int k = l16; k < cnt; k += 16) t += src[k];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+            const double dz = __shfl_sync(kFull, t, 16), pq = __shfl_sync(kFull, t, 0);
             al = cg_ratio(dz, pq);
             if (u.fold == 2) alp = u.alpha_buf[rhs];
         }
@@ -216,42 +288,42 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
     if (act && u.fold == 0 && blockIdx.x == 0 && threadIdx.x == 0) u.alpha_buf[rhs] = s_alpha;
     double acc = 0.0;
     F2 acc2{0.0f, 0.0f};
-    for (int item = threadIdx.x; item < T * TH; item += blockDim.x) {
+    auto update = [&](int item, Item& e) {
         const int c = item % TH, tau = item / TH;
-        const int i = i0 + 2 * c;          // N is even, so i < N implies i + 1 < N
-        R xa = R(0), xb = R(0);
-        if (i < N) {
-            const long o = base + (long)tau * N + i;
-            ld_pair(v + o, xa, xb);
-            if (act) {
-                R qa, qb;
-                ld_pair(u.q + o, qa, qb);
-                if (u.fold != 0) {
-                    R ea, eb, pa, pb;
-                    ld_pair(u.x + o, ea, eb);
-                    ld_pair(u.p + o, pa, pb);
-                    if (u.fold == 2) {
-                        R qa2, qb2;
-                        ld_pair(u.pp + o, qa2, qb2);
-                        ea = fma(ap, qa2, ea);
-                        eb = fma(ap, qb2, eb);
-                    }
-                    ea = fma(al, pa, ea);
-                    eb = fma(al, pb, eb);
-                    st_pair(u.x + o, ea, eb);
+        const long o = offset(item);
+        R xa = e.r[0], xb = e.r[1];
+        if (o >= 0 && act) {
+            if (u.fold != 0) {
+                R ea = e.x[0], eb = e.x[1];
+                if (u.fold == 2) {
+                    ea = fma(ap, e.pp[0], ea);
+                    eb = fma(ap, e.pp[1], eb);
                 }
-                xa = fma(-al, qa, xa);
-                xb = fma(-al, qb, xb);
-                st_pair(v + o, xa, xb);
-                const R part = fma(xa, xa, xb * xb);
-                if constexpr (sizeof(R) == 4)
-                    acc2 = f2_add(acc2, (float)part);
-                else
-                    acc += (double)part;
+                ea = fma(al, e.p[0], ea);
+                eb = fma(al, e.p[1], eb);
+                st_pair(u.x + o, ea, eb);
             }
+            xa = fma(-al, e.q[0], xa);
+            xb = fma(-al, e.q[1], xb);
+            st_pair(v + o, xa, xb);
+            const R part = fma(xa, xa, xb * xb);
+            if constexpr (sizeof(R) == 4)
+                acc2 = f2_add(acc2, (float)part);
+            else
+                acc += (double)part;
         }
         const C2 t = tw<R>(w2, tau, T);    // exp(-i pi tau / T)
         a[tau * TH + c] = Cx<R>::mk(xa * t.x - xb * t.y, xa * t.y + xb * t.x);
+    };
+#pragma unroll
+    for (int k = 0; k < kUpdItems; ++k) {
+        const int item = threadIdx.x + k * 256;
+        if (item < T * TH) update(item, pre[k]);
+    }
+    for (int item = threadIdx.x + kUpdItems * 256; item < T * TH; item += 256) {
+        Item e;
+        load(offset(item), e);
+        update(item, e);
     }
     {
         double sum;
@@ -291,14 +363,22 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
 template <typename R, int TC = 0, int TSC = 0>
 __global__ void __launch_bounds__(256) k_tau_inv(const typename Cx<R>::T2* __restrict__ yh,
                                                  R* __restrict__ y,
-                                                 const typename Cx<R>::T2* __restrict__ w2, int T_,
+                                                 const typename Cx<R>::T2* __restrict__ w2g, int T_,
                                                  int N, int TS_, RadixPlan plan, R scale,
                                                  const R* __restrict__ rdot,
                                                  double* __restrict__ dot_part)
 {
-    pdl_wait();      // the input comes from the previous kernel of the stream
-    const PdlTriggerAtExit pdl_at_exit;
     using C2 = typename Cx<R>::T2;
+    // the twiddles come to shared memory while the previous kernel ends (read
+    // from L2 in every pass they cost each its latency)
+    const C2* w2 = w2g;
+    if constexpr (TC > 0) {
+        __shared__ C2 tws[2 * TC];
+        for (int k = threadIdx.x; k < 2 * TC; k += 256) tws[k] = w2g[k];
+        w2 = tws;
+    }
+    pdl_wait();      // the input comes from the previous kernel of the stream
+    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
     const int T = TC > 0 ? TC : T_;
     const int TS = TSC > 0 ? TSC : TS_;
     const int TH = TS / 2;
@@ -331,6 +411,7 @@ __global__ void __launch_bounds__(256) k_tau_inv(const typename Cx<R>::T2* __res
     const long ob = (long)rhs * T * N;
     const R hs = R(0.5) * scale;           // 1 / sqrt T
     double acc = 0.0;
+    F2 acc2{0.0f, 0.0f};
     for (int item = threadIdx.x; item < T * TH; item += blockDim.x) {
         const int c = item % TH, tau = item / TH;
         const int i = i0 + 2 * c;
@@ -344,22 +425,22 @@ __global__ void __launch_bounds__(256) k_tau_inv(const typename Cx<R>::T2* __res
             if (rdot != nullptr) {
                 R ra, rb;
                 ld_pair(rdot + o, ra, rb);
-                // the pair's two products in R, accumulated in FP64 (one
-                // conversion and one FP64 add per pair: the FP64 pipe is scarce)
-                acc += (double)fma(ya, ra, yb * rb);
+                // the pair's two products in R; the sum as a compensated float
+                // pair in FP32 (some 48 bits on the FP32 pipes, cb.cuh)
+                if constexpr (sizeof(R) == 4)
+                    acc2 = f2_add(acc2, fma(ya, ra, yb * rb));
+                else
+                    acc += fma(ya, ra, yb * rb);
             }
         }
     }
     if (dot_part != nullptr) {
-        __shared__ double red[8];
-        acc = warp_sum(acc);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[k];
-            dot_part[(long)rhs * kRedStride + blockIdx.x] = s;
-        }
+        double sum;
+        if constexpr (sizeof(R) == 4)
+            sum = block_sum_f2(acc2);
+        else
+            sum = block_sum(acc);
+        if (threadIdx.x == 0) dot_part[(long)rhs * kRedStride + blockIdx.x] = sum;
     }
 }
 
