@@ -11,9 +11,9 @@ products, FP64 reliable updates every 50 iterations), and the phonon force
 summed over the 16 solutions.
 
 Metric: CG solves/s (whole job, all ranks); the JSON line also carries
-matvecs/s, the roofline of the dominant kernel (the fused FP32 M^T M of the
-CG iteration, timed live with CUDA events on its stream during the timed
-region), the FP64-only solve rate on the same inputs, the end-to-end rate
+matvecs/s, the roofline of the dominant kernel (by default the whole CG solve
+on chip, one launch per solve; timed live with CUDA events on its stream during
+the timed region), the FP64-only solve rate on the same inputs, the end-to-end rate
 through the public API with host buffers, the clocks seen during the timed
 region, and the oracle timed on the host cores (cpu_baseline).
 
@@ -283,7 +283,12 @@ def run_ours(a):
     torch.cuda.synchronize()
     clocks = Clocks(torch.cuda.current_device())
     clocks.start()
-    ctx.timer_enable(TIMER_STRIDE)
+    # the solve on chip is one launch: every launch is timed; the other loops
+    # launch some five thousand kernels per solve, of which a sample is
+    on_chip = ctx.get_option("resident_cg") and not a.precond and not any(
+        ctx.get_option(o) for o in ("fused_cg", "merged_cg", "persistent_cg"))
+    stride = 1 if on_chip else TIMER_STRIDE
+    ctx.timer_enable(stride)
     l0 = hg.hol_launch_count()
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
@@ -309,6 +314,10 @@ def run_ours(a):
         ctx_kernel_name = ("k_cg_merged (one kernel per CG iteration: p = r + beta p, "
                            "s = w + beta s, x += alpha p every other iteration, "
                            "r' = r - alpha s, w' = M^T M r', r'.r' and |M r'|^2)")
+    elif on_chip and up_cnt == 0:
+        ctx_kernel_name = ("k_cg_resident<float,32> (the whole solve in one launch, one cluster "
+                           "per right-hand side: every vector of the iteration in registers, "
+                           "shared and tensor memory; FP64 true residuals inside)")
     elif op_avg_ms_hint(op_ms, op_cnt, up_cnt):
         ctx_kernel_name = ("k_cg_persist (fused CG chunk: p = r + beta p, q = M^T M p in shared "
                            "memory, e += alpha p, r -= alpha q; per iteration r, p, e read and "
@@ -351,8 +360,23 @@ def run_ours(a):
     # (operator + vector update, every array once) over the wall time per
     # iteration of the timed steps, which also carries the reliable updates,
     # the polling, the set-up, b = M^T R and the force.
-    it_bytes = alg_bytes + (up_units / up_cnt if up_cnt else 0.0)
     it_count = float(np.sum(np.max(iters, axis=1)))   # iterations the loop ran, per step
+    if on_chip and up_cnt == 0:   # HBM moves only inputs and solution: counted per solve
+        # bytes that reach L2 or HBM: b once, and per true residual v read and
+        # written, v and b read, M v written and read (FP64); flops: two applies of
+        # 10 and 12 for the vector updates and sums, per element and iteration
+        nd = float(w.N * w.Ltau)
+        n_rel = float(np.sum(np.ceil(iters / RELIABLE_EVERY))) / a.steps
+        alg_bytes = nd * (n_rel * 48.0 + nr * 8.0)
+        op_units = alg_bytes * op_cnt
+        achieved = op_units / max(op_ms / 1e3, 1e-12) / 1e9
+        solve_flops = nd * 32.0 * float(np.sum(iters)) / a.steps
+        solve_tflops = solve_flops / max(op_avg_ms / 1e3, 1e-12) / 1e12
+        traffic = traffic_from_profiles(ctx_kernel_name.split()[0], op_cnt and alg_bytes)
+        it_bytes = alg_bytes * a.steps / it_count
+    else:
+        solve_flops = solve_tflops = None
+        it_bytes = alg_bytes + (up_units / up_cnt if up_cnt else 0.0)
     it_us = ms_total * 1e3 / it_count
     cg_iteration = {"alg_bytes": it_bytes, "us_per_iteration": it_us,
                     "achieved_gbs": it_bytes / (it_us * 1e-6) / 1e9,
@@ -505,21 +529,28 @@ def run_ours(a):
             "mean_cg_iters": float(np.mean(iters)),
             "tuned_launch": tuned,
             "options": a.option,
-            "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+            "roofline": {"bound": "hbm" if solve_flops is None else
+                         "issue slots and latency on chip (fp32); the hbm fraction only shows "
+                         "that the vectors do not move", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": traffic,
                          "kernel": ctx_kernel_name,
                          "alg_bytes_per_launch": alg_bytes,
                          "avg_launch_ms": op_avg_ms, "launches": op_cnt,
-                         "sampling": f"CUDA events around one launch in {TIMER_STRIDE} of the "
-                                     f"timed region, on the launching stream (warm: the CG "
-                                     f"vectors stay in L2 between launches)",
+                         "fp32": None if solve_flops is None else {
+                             "flops_per_launch": solve_flops, "achieved_tflops": solve_tflops,
+                             "peak_tflops": alu["fp32_fma_gflops"] / 1e3,
+                             "frac": solve_tflops * 1e3 / alu["fp32_fma_gflops"]},
+                         "sampling": f"CUDA events around one launch in {stride} of the "
+                                     f"timed region, on the launching stream"
+                                     + (" (warm: the CG vectors stay in L2 between launches)"
+                                        if solve_flops is None else ""),
                          "peak_src": "MEASURED_PEAKS.json hbm_gbs (of measured)",
                          "cold": cold},
             "cg_iteration": cg_iteration,
             "unit_rates": rates,
             "kernel_ms": {"cg_operator": op_ms, "cg_update": up_ms, "force": fo_ms,
                           "precond": pc_ms, "timed_total": ms_total,
-                          "timer_stride": TIMER_STRIDE,
+                          "timer_stride": stride,
                           "recorded_launches": {"cg_operator": op_cnt, "cg_update": up_cnt,
                                                 "force": fo_cnt, "precond": pc_cnt}},
             "fp64_compare": fp64,
@@ -1148,14 +1179,14 @@ def kernel_source_digest(kernel):
     import re
     name = kernel.split("<")[0]
     # (launch bounds may hold one level of parentheses: sizeof(R) == 4 ? 4 : 2)
-    pat = re.compile(r"__global__ void(?: __launch_bounds__\((?:[^()]|\([^()]*\))*\))? "
+    pat = re.compile(r"__global__ void(?:\s+__launch_bounds__\((?:[^()]|\([^()]*\))*\))?\s+"
                      + re.escape(name) + r"\(")
     csrc = os.path.join(ROOT, "paper_2203_01291_gb300", "csrc")
     h = hashlib.sha256()
     for hname in KERNEL_HEADERS:
         with open(os.path.join(csrc, hname), "rb") as f:
             h.update(f.read())
-    for path in sorted(glob.glob(os.path.join(csrc, "*.cu"))):
+    for path in sorted(glob.glob(os.path.join(csrc, "*.cu"))) + [os.path.join(csrc, "resident.cuh")]:
         src = open(path).read()
         m = pat.search(src)
         if not m:

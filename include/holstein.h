@@ -38,8 +38,9 @@ extern "C" {
 #define HOL_EINVAL   -1   /* bad argument (size, null pointer, unsupported shape) */
 #define HOL_ENOTCONV -2   /* CG did not reach the tolerance within max_iter     */
 #define HOL_ENUMERIC -3   /* NaN / Inf met in a reduction                        */
-#define HOL_ETIMEOUT -4   /* reserved: a bounded device-side wait gave up (no
-                             call of this version waits on the device)          */
+#define HOL_ETIMEOUT -4   /* reserved (the one device-side wait, between the
+                             blocks of a cluster in a solve on chip, is bounded
+                             and ends such a solve with HOL_ENUMERIC)           */
 #define HOL_ECUDA    -5   /* a CUDA runtime call failed                          */
 #define HOL_ENOMEM   -6   /* device allocation failed                            */
 
@@ -161,8 +162,9 @@ typedef struct hol_cg_opts {
  * the residual is replaced by the FP64 true residual; the search direction
  * is then re-conjugated against it, beta = -(z, A p) / (p, A p). The
  * iteration kernels are chosen by the context's launch options (see
- * hol_set_option: two kernels per iteration by default, fused_cg /
- * merged_cg for one).
+ * hol_set_option): without a preconditioner the whole solve is one launch with
+ * its state on chip where that fits (resident_cg, the default); else two
+ * kernels per iteration (fused_cg / merged_cg: one).
  * iters, resid: HOST arrays of n_rhs entries (nullable) receiving the
  * iterations and the final true relative residual of each right-hand side.
  * Returns HOL_ENOTCONV if some right-hand side did not converge (v then holds
@@ -371,16 +373,16 @@ int measure_batch(hol_ctx* const* ctxs, int n_chains, const double* const* xi, i
  *
  * cg_solve_graph: the solve of cg_solve -- the same kernels, the same
  * decisions, so bitwise the same v, iterations and residuals -- with every
- * decision of its loop taken on the device: the loop over chunks of
+ * decision of its loop taken on the device. A solve on chip (resident_cg) is one
+ * kernel node. Otherwise the loop over chunks of
  * check_every iterations is a conditional WHILE node of a CUDA graph, the
  * reliable update (and the certification by the FP64 true residual) a
  * conditional IF node inside it; the host launches the graph once and waits
- * for it. Requires an even check_every and the two-kernel CG iteration
- * (options fused_cg, merged_cg and persistent_cg off), else HOL_EINVAL. The
- * loop runs whole chunks: with max_iter not a multiple of check_every it can
+ * for it. Requires an even check_every and the options fused_cg, merged_cg and
+ * persistent_cg off, else HOL_EINVAL. The WHILE loop runs whole chunks: with max_iter not a multiple of check_every it can
  * run up to check_every - 1 iterations past max_iter before HOL_ENOTCONV; the
- * number of chunks is bounded by max_iter / check_every + 2 in every case (no
- * device-side wait exists that could hang). Arguments and results as
+ * number of chunks is bounded by max_iter / check_every + 2 in every case. A
+ * solve on chip stops at max_iter. Arguments and results as
  * cg_solve; uses the context's scratch and internal streams; synchronises
  * `stream`.
  *
