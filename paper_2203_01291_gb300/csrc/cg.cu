@@ -125,8 +125,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_cg_update(R* __
         // in every warp measured slower than the barrier)
         __shared__ double s_alpha, s_alpha_prev;
         if (threadIdx.x < 32) {
-            const double pq = warp_sum_array(pq_part + (long)rhs * pq_stride, pq_n);
-            const double dz = warp_sum_array(dz_part + (long)rhs * kRedStride, dz_n);
+            const double2 sums = warp_sum_pair(pq_part + (long)rhs * pq_stride, pq_n,
+                                               dz_part + (long)rhs * kRedStride, dz_n);
+            const double pq = sums.x, dz = sums.y;
             if (threadIdx.x == 0) {
                 s_alpha = cg_ratio(dz, pq);
                 if (FOLD == 2) s_alpha_prev = alpha_buf[rhs];

@@ -361,9 +361,9 @@ __global__ void __launch_bounds__(128, 2) k_cg_mtm32_v4s(const float* __restrict
         const long base = (long)rhs * gm.T * N;
         float bt = 0.0f;
         if (!first) {
-            const double rn = warp_sum_array(rr_new_part + (long)rhs * rr_stride, rr_n);
-            const double ro = warp_sum_array(rr_old_part + (long)rhs * rr_stride, rr_n);
-            bt = (float)cg_ratio(rn, ro);
+            const double2 rr = warp_sum_pair(rr_new_part + (long)rhs * rr_stride, rr_n,
+                                             rr_old_part + (long)rhs * rr_stride, rr_n);
+            bt = (float)cg_ratio(rr.x, rr.y);
         }
         float4 W[RT], X[RT], P[RT], Y[RT];
         issue(pos + S - 1);
@@ -648,9 +648,9 @@ __global__ void __launch_bounds__(32 * NW) k_cg_mtm32_split(const float* __restr
         }
         float bt = 0.0f;
         if (!first) {
-            const double rn = warp_sum_array(rr_new_part + (long)rhs * rr_stride, rr_n);
-            const double ro = warp_sum_array(rr_old_part + (long)rhs * rr_stride, rr_n);
-            bt = (float)cg_ratio(rn, ro);
+            const double2 rr = warp_sum_pair(rr_new_part + (long)rhs * rr_stride, rr_n,
+                                             rr_old_part + (long)rhs * rr_stride, rr_n);
+            bt = (float)cg_ratio(rr.x, rr.y);
         }
         if (threadIdx.x == 0) s_bt = bt;
     }

@@ -61,9 +61,9 @@ __device__ __forceinline__ float cg_beta(const MvGeom& gm, int rhs, int first,
 {
     if (first) return 0.0f;
     if (gm.beta_in != nullptr) return (float)gm.beta_in[rhs];
-    const double rn = warp_sum_array(rr_new_part + (long)rhs * rr_stride, rr_n);
-    const double ro = warp_sum_array(rr_old_part + (long)rhs * rr_stride, rr_n);
-    return (float)cg_ratio(rn, ro);
+    const double2 rr = warp_sum_pair(rr_new_part + (long)rhs * rr_stride, rr_n,
+                                     rr_old_part + (long)rhs * rr_stride, rr_n);
+    return (float)cg_ratio(rr.x, rr.y);
 }
 
 // CG operator epilogue: once every warp of a right-hand side has stored its
@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(128) k_M(const R* __restrict__ v, const R* __r
     const long base = (long)rhs * gm.T * N + geo.ix;
     R bt = R(0);
     if (UPD && !bsrc.first) {
-        const double rn = warp_sum_array(bsrc.rn + (long)rhs * bsrc.stride, bsrc.n);
-        const double ro = warp_sum_array(bsrc.ro + (long)rhs * bsrc.stride, bsrc.n);
-        bt = (R)cg_ratio(rn, ro);
+        const double2 rr = warp_sum_pair(bsrc.rn + (long)rhs * bsrc.stride, bsrc.n,
+                                         bsrc.ro + (long)rhs * bsrc.stride, bsrc.n);
+        bt = (R)cg_ratio(rr.x, rr.y);
     }
 
     R a[L], c[L];

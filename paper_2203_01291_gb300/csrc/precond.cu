@@ -108,7 +108,7 @@ __device__ __forceinline__ void st_cpair(double2* p, double2 a, double2 b)
 // (fft.cuh), and the joined update and the r.z sum stay off the FP64 pipe.
 // P^{-1} P^{-T}, L = 16, Ltau = 160, 2 rhs: 15.2 -> 13.8 us; L = 32, Ltau = 200,
 // 16 rhs: 48.4 -> 40; a preconditioned iteration at L = 16, Ltau = 160, 2 rhs, all
-// kernels: 27.6 -> 24.5 us.
+// kernels: 27.6 -> 24.5 us (22.5 with the paired sums of alpha and beta, cb.cuh).
 template <bool EARLY>
 struct PdlTriggerFp32 {
     __device__ __forceinline__ PdlTriggerFp32() { if (EARLY) pdl_trigger(); }
@@ -265,17 +265,9 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
     if (threadIdx.x < 32) {
         double al = 0.0, alp = 0.0;
         if (act) {
-            // the two sums in the two halves of the warp
-            const int half = threadIdx.x >> 4, l16 = threadIdx.x & 15;
-            const double* src = half ? u.dz_part + (long)rhs * kRedStride
-                                     : u.pq_part + (long)rhs * u.pq_stride;
-            const int cnt = half ? u.dz_n : u.pq_n;
-            double t = 0.0;
-            for (int k = l16; k < cnt; k += 16) t += src[k];
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-            const double dz = __shfl_sync(kFull, t, 16), pq = __shfl_sync(kFull, t, 0);
-            al = cg_ratio(dz, pq);
+            const double2 sums = warp_sum_pair(u.pq_part + (long)rhs * u.pq_stride, u.pq_n,
+                                               u.dz_part + (long)rhs * kRedStride, u.dz_n);
+            al = cg_ratio(sums.y, sums.x);
             if (u.fold == 2) alp = u.alpha_buf[rhs];
         }
         if (threadIdx.x == 0) {
