@@ -17,10 +17,11 @@
 //   (relative error of a series, mean over seven shapes: 6.4e-7, 1.1e-6 with
 //   one float or with the older kernels' unfolded constants). P^{-1} P^{-T} at
 //   L = 16, Ltau = 160 on 2 rhs 15.2 us (30.4 with the one-column layout
-//   k_kpm_lane); 13.8 with the set-up ahead of the wait for the forward transform.
+//   k_kpm_lane); 14.2 with the set-up ahead of the wait for the forward transform.
 //   k_kpm_rows (FP32, L >= 20): the strip over several warps per part, since one
 //   warp's issue slots would bound a step (L = 32: 500 cycles); one exchange of
-//   edge rows per step. L = 32, Ltau = 200: 24.7 us on 2 rhs (41.0 with k_kpm_reg).
+//   edge rows per step. L = 32, Ltau = 200: 23.2 us on 2 rhs (42.2 with
+//   k_kpm_reg), 40.0 on 16 (57.7).
 //   k_kpm_pair (FP64): a step is bound by the FP64 pipe (an FP64 instruction
 //   holds its quarter of a multiprocessor for sixty cycles), so a problem's two
 //   parts take one multiprocessor each (a cluster of two blocks) and a part is

@@ -106,7 +106,7 @@ __device__ __forceinline__ void st_cpair(double2* p, double2 a, double2 b)
 // input, a barrier and a trip through shared memory per pass, the sums. So the
 // twiddles wait in shared memory, an odd power of two takes a radix 8 pass
 // (fft.cuh), and the joined update and the r.z sum stay off the FP64 pipe.
-// P^{-1} P^{-T}, L = 16, Ltau = 160, 2 rhs: 15.2 -> 13.8 us; L = 32, Ltau = 200,
+// P^{-1} P^{-T}, L = 16, Ltau = 160, 2 rhs: 15.2 -> 14.2 us; L = 32, Ltau = 200,
 // 16 rhs: 48.4 -> 40; a preconditioned iteration at L = 16, Ltau = 160, 2 rhs, all
 // kernels: 27.6 -> 24.5 us (22.5 with the paired sums of alpha and beta, cb.cuh).
 template <bool EARLY>
