@@ -320,9 +320,11 @@ extern "C" int hol_create(const hol_params* p, hol_ctx** out)
     }
     if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) !=
             cudaSuccess ||
-        c->sms < 1) {
+        c->sms < 1 ||
+        cudaDeviceGetAttribute(&c->smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) !=
+            cudaSuccess) {
         free_ctx(c);
-        return set_error(HOL_ECUDA, "hol_create: multiprocessor count query failed");
+        return set_error(HOL_ECUDA, "hol_create: device attribute query failed");
     }
     if (c->exact)
         occ64_warm_exact(c);

@@ -174,6 +174,7 @@ struct hol_ctx {
     long n;              // N * T
     int device;
     int sms;             // streaming multiprocessors of the device
+    int smem_max;        // most shared memory of one block
     double th;           // tanh(dtau t): checkerboard bond [[1, th], [th, 1]]
     double ch4;          // cosh(dtau t)^4, folded into the stored exp(-dtau V)
                          // (1 with the exact propagator)

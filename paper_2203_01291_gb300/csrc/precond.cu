@@ -1278,6 +1278,14 @@ __global__ void __launch_bounds__(KBand<L>::THREADS > 0 ? KBand<L>::THREADS : 32
 // coefficient is N_P terms of two multiply-adds, four lanes per coefficient. (A
 // rotation per term over all N_Q nodes took six FP64 operations each, 27 us at
 // Ltau = 160 on the FP64 pipe's sixty cycles an instruction; now 8.4.)
+// LONG: node sums and table no longer fit beside each other. An even m reads only the
+// even sums and the even entries of the table, an odd m the odd ones, so the
+// parities take turns in one array of either (24 bytes per order instead of 48)
+// at the price of evaluating the nodes twice. Field set-up in all at L = 4: 139 us
+// at Ltau = 1200 (both parities at once), 154 at 1250 (in turn); the rotations took
+// 488 and 510.
+constexpr size_t kCoefStatic = 64;   // its static shared memory, rounded up
+template <bool LONG>
 __global__ void __launch_bounds__(256) k_kpm_coeffs(const double* __restrict__ scal, int T, int max_np,
                                                     int* __restrict__ npv, double2* __restrict__ coef,
                                                     float4* __restrict__ coef32,
@@ -1287,7 +1295,7 @@ __global__ void __launch_bounds__(256) k_kpm_coeffs(const double* __restrict__ s
 {
     pdl_wait();      // the bounds come from the previous kernel of the stream
     const PdlTriggerAtExit pdl_at_exit;
-    extern __shared__ double2 fq[];              // [2][max_np] even, odd sums; then the table
+    extern __shared__ double2 fq[];   // even, odd sums [2][max_np] (LONG: of one parity), then the table
     const int w = blockIdx.x;
     const double bmin = scal[S_BMIN], bmax = scal[S_BMAX];
     const double db = bmax - bmin;
@@ -1317,11 +1325,6 @@ __global__ void __launch_bounds__(256) k_kpm_coeffs(const double* __restrict__ s
     __syncthreads();
     const int np = s_np, nq = 2 * np;
     const double inv = s_inv, sp = s_sin, cp = s_cos;
-    double2* fe = fq;
-    double2* fo = fq + max_np;
-    double* ct = reinterpret_cast<double*>(fq + 2 * max_np);   // [2 max_np + 1]
-    for (int k = threadIdx.x; k <= nq; k += blockDim.x) ct[k] = cospi(k * inv);
-    __syncthreads();
     // f = 1 / (1 - e^{-i phi} bb) = 1 / ((1 - bb cos phi) + i bb sin phi) at the
     // nodes +-y
     auto node = [&](double y) -> double2 {
@@ -1330,47 +1333,72 @@ __global__ void __launch_bounds__(256) k_kpm_coeffs(const double* __restrict__ s
         const double iden = 1.0 / (re * re + im * im);
         return make_double2(re * iden, -im * iden);
     };
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {   // nodes q < np, then their mirrors
-        const int p = q < np ? q : q - np;
-        const double y = ct[2 * p + 1];
-        (q < np ? fe : fo)[p] = node(q < np ? y : -y);
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < np; q += blockDim.x) {
-        const double2 u = fe[q], v = fo[q];
-        fe[q] = make_double2(u.x + v.x, u.y + v.y);
-        fo[q] = make_double2(u.x - v.x, u.y - v.y);
-    }
-    __syncthreads();
-    const int sub = threadIdx.x & 3;
-    for (int m0 = 0; m0 < np; m0 += blockDim.x / 4) {
-        const int m = m0 + (threadIdx.x >> 2);
-        double sr = 0.0, si = 0.0;
-        if (m < np) {
-            const double2* f = (m & 1) ? fo : fe;
-            int k = (int)((long)m * (2 * sub + 1) % (4 * nq));
-            const int step = (int)((long)m * 8 % (4 * nq));
-            for (int q = sub; q < np; q += 4) {
-                const int kk = k > 2 * nq ? 4 * nq - k : k;
-                const double c = kk > nq ? -ct[2 * nq - kk] : ct[kk];
-                const double2 fv = f[q];
-                sr = fma(c, fv.x, sr);
-                si = fma(c, fv.y, si);
-                k += step;
-                if (k >= 4 * nq) k -= 4 * nq;
+    // c_m, m = first, first + inc, ...; entry k of the table at ct[k / inc]
+    constexpr int inc = LONG ? 2 : 1;
+    auto coeffs = [&](const double2* fe, const double2* fo, const double* ct, int first) {
+        const int sub = threadIdx.x & 3;
+        for (int m0 = first; m0 < np; m0 += inc * (int)(blockDim.x / 4)) {
+            const int m = m0 + inc * (int)(threadIdx.x >> 2);
+            double sr = 0.0, si = 0.0;
+            if (m < np) {
+                const double2* f = (m & 1) ? fo : fe;
+                int k = (int)((long)m * (2 * sub + 1) % (4 * nq));
+                const int step = (int)((long)m * 8 % (4 * nq));
+                for (int q = sub; q < np; q += 4) {
+                    const int kk = k > 2 * nq ? 4 * nq - k : k;
+                    const double c = kk > nq ? -ct[(2 * nq - kk) / inc] : ct[kk / inc];
+                    const double2 fv = f[q];
+                    sr = fma(c, fv.x, sr);
+                    si = fma(c, fv.y, si);
+                    k += step;
+                    if (k >= 4 * nq) k -= 4 * nq;
+                }
+            }
+#pragma unroll
+            for (int o = 2; o > 0; o >>= 1) {
+                sr += __shfl_xor_sync(kFull, sr, o);
+                si += __shfl_xor_sync(kFull, si, o);
+            }
+            if (m < np && sub == 0) {
+                const double fac = m == 0 ? 2.0 * inv : 4.0 * inv;   // pi / (q_m N_Q)
+                const double cr = fac * sr, ci = fac * si;
+                coef[(long)w * max_np + m] = make_double2(cr, ci);
+                coef32[(long)w * max_np + m] = make_float4((float)cr, (float)cr, (float)ci, (float)ci);
             }
         }
-#pragma unroll
-        for (int o = 2; o > 0; o >>= 1) {
-            sr += __shfl_xor_sync(kFull, sr, o);
-            si += __shfl_xor_sync(kFull, si, o);
+    };
+    if constexpr (LONG) {
+        double* ct = reinterpret_cast<double*>(fq + max_np);   // [max_np + 1]
+        for (int par = 0; par < 2; ++par) {
+            for (int k = threadIdx.x; 2 * k + par <= nq; k += blockDim.x) ct[k] = cospi((2 * k + par) * inv);
+            for (int q = threadIdx.x; q < np; q += blockDim.x) {
+                const double y = cospi((2 * q + 1) * inv);
+                const double2 u = node(y), v = node(-y);
+                fq[q] = par ? make_double2(u.x - v.x, u.y - v.y) : make_double2(u.x + v.x, u.y + v.y);
+            }
+            __syncthreads();
+            coeffs(fq, fq, ct, par);
+            __syncthreads();
         }
-        if (m < np && sub == 0) {
-            const double fac = m == 0 ? 2.0 * inv : 4.0 * inv;   // pi / (q_m N_Q)
-            const double cr = fac * sr, ci = fac * si;
-            coef[(long)w * max_np + m] = make_double2(cr, ci);
-            coef32[(long)w * max_np + m] = make_float4((float)cr, (float)cr, (float)ci, (float)ci);
+    } else {
+        double2* fe = fq;
+        double2* fo = fq + max_np;
+        double* ct = reinterpret_cast<double*>(fq + 2 * max_np);   // [2 max_np + 1]
+        for (int k = threadIdx.x; k <= nq; k += blockDim.x) ct[k] = cospi(k * inv);
+        __syncthreads();
+        for (int q = threadIdx.x; q < nq; q += blockDim.x) {   // nodes q < np, then their mirrors
+            const int p = q < np ? q : q - np;
+            const double y = ct[2 * p + 1];
+            (q < np ? fe : fo)[p] = node(q < np ? y : -y);
         }
+        __syncthreads();
+        for (int q = threadIdx.x; q < np; q += blockDim.x) {
+            const double2 u = fe[q], v = fo[q];
+            fe[q] = make_double2(u.x + v.x, u.y + v.y);
+            fo[q] = make_double2(u.x - v.x, u.y - v.y);
+        }
+        __syncthreads();
+        coeffs(fe, fo, ct, 0);
     }
     const double s4 = s_s4;
     for (int i = w * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
@@ -1706,10 +1734,15 @@ int precond_alloc(hol_ctx* c)
 
 int kpm_setup(hol_ctx* c, cudaStream_t s)
 {
-    const size_t sm = 2 * (size_t)c->kpm.max_np * sizeof(double2) +
-                      (2 * (size_t)c->kpm.max_np + 1) * sizeof(double);
-    if (int rc = smem_raise((const void*)k_kpm_coeffs, sm)) return rc;
-    HOL_CUDA(launch_pdl(c, k_kpm_coeffs, c->T / 2, 256, sm, s, c->scal, c->T, c->kpm.max_np, c->kpm.np,
+    const size_t sums = 2 * (size_t)c->kpm.max_np * sizeof(double2);
+    const size_t table = (2 * (size_t)c->kpm.max_np + 1) * sizeof(double);
+    // both parities at once while sums and table fit (Ltau <= 1206), beyond that in
+    // turn in the room of the sums
+    const bool both = sums + table + kCoefStatic <= (size_t)c->smem_max;
+    const size_t sm = both ? sums + table : sums - kCoefStatic;
+    const auto fn = both ? k_kpm_coeffs<false> : k_kpm_coeffs<true>;
+    if (int rc = smem_raise((const void*)fn, sm)) return rc;
+    HOL_CUDA(launch_pdl(c, fn, c->T / 2, 256, sm, s, c->scal, c->T, c->kpm.max_np, c->kpm.np,
                         c->kpm.coef, c->kpm.coef32, c->dbar, c->N, c->kpm.dk64, c->kpm.dk32,
                         c->kpm.np + c->T / 2, c->kpm_a1, c->kpm_a2));
     HOL_CHECK_LAUNCH("k_kpm_coeffs");
