@@ -20,6 +20,9 @@
 // an iteration crosses the cluster once: two sums per block and two boundary
 // slices, all asynchronous and awaited together.
 //
+// Scale. The iteration runs on b over a power of two near |b| (pow2_hi), so it
+// takes the same steps whatever the scale of b.
+//
 // Control. After every check_every iterations the recursive residual is
 // compared with tol; at tol, or after reliable_every iterations, x is folded
 // into the FP64 solution and r is replaced by the FP64 true residual (the
@@ -337,6 +340,13 @@ __device__ __forceinline__ bool mb_wait(unsigned mb, int parity)
     return false;
 }
 
+// A right-hand side is solved as b / 2^ex, ex the exponent of |b|, so that the FP32
+// sums and their reciprocals stay in range whatever the scale of b. Every vector on
+// chip and v between segments are on that scale; v goes back to b's with the last
+// segment. All exact. The exponent is kept as a difference of high words, ex << 20.
+__device__ __forceinline__ unsigned exp_hi(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) - 0x3ff00000u; }
+__device__ __forceinline__ double pow2_hi(unsigned xs) { return __hiloint2double((int)(0x3ff00000u + xs), 0); }
+
 // FP32 <-> FP64 on the integer pipes for the usual exponents: a conversion
 // instruction takes the FP64 pipe as long as an addition. Same values (round to
 // nearest even); zeros, subnormals, infinities and NaN take the instruction.
@@ -474,6 +484,10 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
     __shared__ int s_stop;                // 1: end of the segment, 2: not finite
     __shared__ __align__(8) unsigned long long s_mb[2];
     __shared__ int s_item;
+    // |b|, (tol |b|)^2 on the scale of r, the exponent of |b| (pow2_hi): of the item in
+    // hand, here and not in registers of the iteration
+    __shared__ double s_bnorm, s_limit;
+    __shared__ unsigned s_bxs;
     __shared__ unsigned s_tm;
 
     const int t0 = (int)((long)a.T * crank / cs), t1 = (int)((long)a.T * (crank + 1) / cs);
@@ -768,7 +782,6 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
     int item = -1;          // right-hand side in hand (uniform over the cluster)
     bool loaded = false;    // its r and p are on chip
     int it = 0;
-    double bnorm = 0.0;
     for (;;) {
         // ------------------------------------------------ the next segment's item
         if (crank == 0 && wid == 0) {
@@ -827,7 +840,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
             cl.sync();
             if (crank == 0 && threadIdx.x == 0) {
                 a.d.it[item] = it;
-                a.d.bnorm[item] = bnorm;
+                a.d.bnorm[item] = s_bnorm;
                 __threadfence();
                 atomicExch(a.d.rstate + item, RS_READY);
             }
@@ -839,46 +852,20 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         const long rbase = (long)item * a.T * N, base = rbase + (long)t0 * N;
         if (!loaded) {
             it = __ldcg(a.d.it + item);
-            bnorm = __ldcg(a.d.bnorm + item);
-            double bb = 0.0;
+            double bnorm = __ldcg(a.d.bnorm + item);
+            if (it == 0) {
+                double bb = 0.0;
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                R p[E];
-                const long o = rbase + (held(k) ? (long)tau_of(slice(k)) * N : 0L);
+                for (int k = 0; k < K; ++k)
+                    if (own(k))
 #pragma unroll
-                for (int q = 0; q < RT; ++q) {
-                    V2 tr, tq;
-                    tr.x = tr.y = tq.x = tq.y = R(0);
-                    if (held(k) && geo.has(q)) {
-                        if (it == 0) {
-                            const double2 t = *reinterpret_cast<const double2*>(a.b + o + geo.site(q));
-                            if (own(k)) {
+                        for (int q = 0; q < RT; ++q)
+                            if (geo.has(q)) {
+                                const double2 t = *reinterpret_cast<const double2*>(
+                                    a.b + base + (long)slice(k) * N + geo.site(q));
                                 bb = fma(t.x, t.x, bb);
                                 bb = fma(t.y, t.y, bb);
                             }
-                            tr.x = from_f64<R>(t.x);
-                            tr.y = from_f64<R>(t.y);
-                        } else {
-                            tr = __ldcg(reinterpret_cast<const V2*>(rsave + o + geo.site(q)));
-                            tq = __ldcg(reinterpret_cast<const V2*>(psave + o + geo.site(q)));
-                        }
-                    }
-                    r[k][2 * q] = tr.x; r[k][2 * q + 1] = tr.y;
-                    p[2 * q] = tq.x; p[2 * q + 1] = tq.y;
-                }
-                if constexpr (TM) {
-#pragma unroll
-                    for (int e = 0; e < E; e += CH) {
-                        R u[CH];
-#pragma unroll
-                        for (int q = 0; q < CH; ++q) u[q] = p[e + q];
-                        tm_st<CH>(tp(k, e), u);
-                    }
-                } else {
-                    if (own(k)) slot_st<R, L>(ps + (long)slice(k) * SL, geo.ll, p);
-                }
-            }
-            if (it == 0) {
                 bnorm = sqrt(reduce64(bb));
                 if (bnorm == 0.0 || !isfinite(bnorm)) {   // v = 0 is exact, or nothing is
 #pragma unroll
@@ -903,6 +890,49 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                     }
                     item = -1;
                     continue;
+                }
+            }
+            const unsigned bxs = exp_hi(bnorm);
+            if (threadIdx.x == 0) {
+                // a tolerance far below the FP64 rounding of b still folds before the
+                // sums leave their range
+                const double tb = a.tol * (bnorm * pow2_hi(0u - bxs));
+                s_bnorm = bnorm;
+                s_limit = fmax(tb * tb, sizeof(R) == 4 ? 1e-34 : 1e-290);
+                s_bxs = bxs;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                R p[E];
+                const long o = rbase + (held(k) ? (long)tau_of(slice(k)) * N : 0L);
+#pragma unroll
+                for (int q = 0; q < RT; ++q) {
+                    V2 tr, tq;
+                    tr.x = tr.y = tq.x = tq.y = R(0);
+                    if (held(k) && geo.has(q)) {
+                        if (it == 0) {
+                            const double2 t = *reinterpret_cast<const double2*>(a.b + o + geo.site(q));
+                            tr.x = from_f64<R>(t.x * pow2_hi(0u - bxs));
+                            tr.y = from_f64<R>(t.y * pow2_hi(0u - bxs));
+                        } else {
+                            tr = __ldcg(reinterpret_cast<const V2*>(rsave + o + geo.site(q)));
+                            tq = __ldcg(reinterpret_cast<const V2*>(psave + o + geo.site(q)));
+                        }
+                    }
+                    r[k][2 * q] = tr.x; r[k][2 * q + 1] = tr.y;
+                    p[2 * q] = tq.x; p[2 * q + 1] = tq.y;
+                }
+                if constexpr (TM) {
+#pragma unroll
+                    for (int e = 0; e < E; e += CH) {
+                        R u[CH];
+#pragma unroll
+                        for (int q = 0; q < CH; ++q) u[q] = p[e + q];
+                        tm_st<CH>(tp(k, e), u);
+                    }
+                } else {
+                    if (own(k)) slot_st<R, L>(ps + (long)slice(k) * SL, geo.ll, p);
                 }
             }
             loaded = true;
@@ -972,7 +1002,6 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         AT gpart = own_dot(r, r);
 
         // ------------------------------------------------ iterations
-        const double limit = (a.tol * bnorm) * (a.tol * bnorm);
         int since = 0;
         bool bad = false;
         for (;;) {
@@ -982,7 +1011,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
             reduce(gamma, delta);
             if (wid == 0) {
                 // |r| / |b| < tol, as gamma against (tol |b|)^2
-                const int stop = lost ? 2 : since > 0 && since % a.chk == 0 ? A::stop(gamma, limit) : 0;
+                const int stop = lost ? 2 : since > 0 && since % a.chk == 0 ? A::stop(gamma, s_limit) : 0;
                 R al, be;
                 st.step(gamma, delta, given, beta0, corr, al, be);
                 if (lane == 0) {
@@ -1060,6 +1089,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         // every block has read its exchange slots and s: the FP64 exchange takes
         // their place. v += x, C v to the successor
         cl.sync();
+        const double down = pow2_hi(0u - s_bxs);
         double* const ex64_next0 = cl.map_shared_rank(ex64, next);
         double* const ex64_prevn = cl.map_shared_rank(ex64, prev) + (long)prev_nc * SL;
         if constexpr (TM) tm_stored();
@@ -1131,7 +1161,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                         const double wx = fma(dx, tq[0], u[q].x), wy = fma(dy, tq[1], u[q].y);
                         if (geo.has(q0 + q))
                             __stcg(reinterpret_cast<double2*>(a.t64 + o + geo.site(q0 + q)),
-                                   make_double2(bv[q].x - wx, bv[q].y - wy));
+                                   make_double2(fma(bv[q].x, down, -wx), fma(bv[q].y, down, -wy)));
                         tq[0] = dx * wx;
                         tq[1] = dy * wy;
                     }
@@ -1169,12 +1199,27 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
             }
             halo_send(k, r[k], false);
         }
-        const double tres = sqrt(reduce64(tr)) / bnorm;
+        const double tres = sqrt(reduce64(tr)) / (s_bnorm * pow2_hi(0u - s_bxs));
 #pragma unroll
         for (int k = 0; k < K; ++k) halo_recv(k, hpar, r[k], false);
         hpar ^= 1;
         bad = bad || !isfinite(tres);
         if (bad || tres < a.tol || it >= a.max_iter) {
+            const unsigned bxs = s_bxs;
+            if (bxs != 0)   // v on the scale of b
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (own(k))
+#pragma unroll
+                        for (int q = 0; q < RT; ++q)
+                            if (geo.has(q)) {
+                                double2* vq = reinterpret_cast<double2*>(
+                                    a.v + base + (long)slice(k) * N + geo.site(q));
+                                double2 u = __ldcg(vq);
+                                u.x *= pow2_hi(bxs);
+                                u.y *= pow2_hi(bxs);
+                                __stcg(vq, u);
+                            }
             if (crank == 0 && threadIdx.x == 0) {
                 const bool ok = !bad && tres < a.tol;
                 a.d.it[item] = it;
