@@ -144,8 +144,8 @@ typedef struct hol_cg_opts {
     int max_iter;        /* iteration cap per right-hand side                  */
     int precond;         /* 0: plain CG; 1: adiabatic preconditioner (Sec. VI) */
     int prec;            /* HOL_F64: all FP64. HOL_F32: FP32 matvecs and
-                            iterations, FP64 dot products, FP64 solution and
-                            true-residual (reliable) updates                   */
+                            iterations, dot products compensated (below), FP64
+                            solution and true-residual (reliable) updates      */
     int reliable_every;  /* HOL_F32: iterations between FP64 residual updates  */
     int check_every;     /* iterations between host convergence polls          */
 } hol_cg_opts;
@@ -156,8 +156,10 @@ typedef struct hol_cg_opts {
  * the preconditioner z = P^{-1} P^{-T} r when opts->precond (Eq. (CG_precon)).
  * b, v: FP64 [n_rhs][T][N] (device). Convergence of every right-hand side is
  * certified with an FP64 true residual |b - M^T M v| / |b| < tol. With
- * opts->prec HOL_F32 the iterations run in FP32 (FP64 dot products) and
- * every reliable_every iterations, and whenever the recursive residual
+ * opts->prec HOL_F32 the iterations run in FP32 (dot products: FP32 within a
+ * group of four products, for |M p|^2 within a thread's share of a slice; the groups'
+ * sums as compensated float pairs of some 48 bits, over blocks FP64 in the iteration
+ * kernels and pairs in a solve on chip) and every reliable_every iterations, and whenever the recursive residual
  * estimate falls below tol, the FP32 increment is folded into the FP64 v and
  * the residual is replaced by the FP64 true residual; the search direction
  * is then re-conjugated against it, beta = -(z, A p) / (p, A p). The
