@@ -47,3 +47,30 @@ def test_first_step_length(L, T, every, on):
         ctx.cg_solve(b, v, tol=1e-12, max_iter=1, prec=hg.HOL_F32, raise_on_nonconv=False)
         got = v.reshape(T, L, L)[:, ::every]
         assert float((got / alpha - 1.0).abs().max()) < 2.1e-7
+
+
+@pytest.mark.parametrize("on", [1, 0])
+@pytest.mark.parametrize("prec,tol,rel", [(hg.HOL_F64, 1e-10, 50), (hg.HOL_F32, 1e-5, 100000)])
+@pytest.mark.parametrize("L,T", [(4, 40), (6, 30), (8, 24)])
+def test_check_after_the_first_one_below_tol(L, T, prec, tol, rel, on):
+    """A solve ends at the check after the first one whose residual is below tol: capped one
+    interval earlier, where the cap forces the true residual, it is certified already.
+    In FP32 a single segment (tol above its drift from the true residual), so the
+    recursive residual decides there too; it is the true one but for its drift, 1e-7 of |b|
+    at most, so it may be above tol by that."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(100 + L)
+    with hg.Context(L=L, Ltau=T, alpha=1.0, max_rhs=1) as ctx:
+        ctx.set_option("resident_cg", on)
+        ctx.set_field(torch.randn(T, L * L, dtype=torch.float64, device=DEV, generator=g))
+        for _ in range(5):
+            R = torch.randn(1, T, L * L, dtype=torch.float64, device=DEV, generator=g)
+            b, v = torch.empty_like(R), torch.empty_like(R)
+            ctx.fermion_matvec(hg.HOL_OP_MT, R, b)
+            kw = dict(tol=tol, prec=prec, check_every=10, reliable_every=rel)
+            it, _ = ctx.cg_solve(b, v, **kw)
+            drift = 1e-7 if prec == hg.HOL_F32 else 1e-13
+            _, res = ctx.cg_solve(b, v, max_iter=int(it[0]) - 10, raise_on_nonconv=False, **kw)
+            assert res[0] < tol + drift
+            _, res = ctx.cg_solve(b, v, max_iter=int(it[0]) - 20, raise_on_nonconv=False, **kw)
+            assert res[0] > tol - drift
