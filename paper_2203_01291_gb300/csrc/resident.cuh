@@ -788,6 +788,16 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         return acc;
     };
 
+    // the failure flags of the solve: of several clusters' failures a number that is not
+    // finite counts over a missed tolerance, whichever comes last
+    static_assert(HOL_ENUMERIC < HOL_ENOTCONV && HOL_ENOTCONV < 0, "the code that counts is the lower one");
+    auto fail = [&](int code, int rhs) {
+        if (code != HOL_ENOTCONV) {
+            a.d.g[DCG_ERR_RHS] = rhs;   // one failing rhs (any); reported only
+            atomicMin(&a.d.g[DCG_ERR], code);
+        }
+        atomicMin(&a.d.g[DCG_STICKY], code);
+    };
     int item = -1;          // right-hand side in hand (uniform over the cluster)
     bool loaded = false;    // its r and p are on chip
     int it = 0;
@@ -891,11 +901,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                         a.d.tres[item] = z ? 0.0 : bnorm;
                         a.d.done[item] = z;
                         a.d.rstate[item] = RS_DONE;
-                        if (!z) {
-                            a.d.g[DCG_ERR_RHS] = item;
-                            a.d.g[DCG_ERR] = HOL_ENUMERIC;
-                            a.d.g[DCG_STICKY] = HOL_ENUMERIC;
-                        }
+                        if (!z) fail(HOL_ENUMERIC, item);
                     }
                     item = -1;
                     continue;
@@ -1247,13 +1253,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 a.d.tres[item] = tres;
                 a.d.done[item] = ok;
                 a.d.rstate[item] = RS_DONE;
-                if (!ok) {
-                    if (bad) {
-                        a.d.g[DCG_ERR_RHS] = item;
-                        a.d.g[DCG_ERR] = HOL_ENUMERIC;
-                    }
-                    a.d.g[DCG_STICKY] = bad ? HOL_ENUMERIC : HOL_ENOTCONV;
-                }
+                if (!ok) fail(bad ? HOL_ENUMERIC : HOL_ENOTCONV, item);
             }
             item = -1;
         }
