@@ -38,9 +38,9 @@ extern "C" {
 #define HOL_EINVAL   -1   /* bad argument (size, null pointer, unsupported shape) */
 #define HOL_ENOTCONV -2   /* CG did not reach the tolerance within max_iter     */
 #define HOL_ENUMERIC -3   /* NaN / Inf met in a reduction                        */
-#define HOL_ETIMEOUT -4   /* reserved (the one device-side wait, between the
-                             blocks of a cluster in a solve on chip, is bounded
-                             and ends such a solve with HOL_ENUMERIC)           */
+#define HOL_ETIMEOUT -4   /* a bounded device-side wait gave up (the one between
+                             the blocks of a cluster in a solve on chip, option
+                             resident_wait_ms)                                  */
 #define HOL_ECUDA    -5   /* a CUDA runtime call failed                          */
 #define HOL_ENOMEM   -6   /* device allocation failed                            */
 
@@ -538,6 +538,12 @@ int hol_tune(hol_ctx* ctx, int n_rhs, int* best_k, int* best_warps, int* best_ve
  *                       fits (FP32 iterations: N Ltau up to about 230,000 at
  *                       L = 32; FP64: small systems); 0: the iteration
  *                       kernels below (0/1, default 1)
+ *   "resident_wait_ms"  longest wait of a block of such a cluster for the
+ *                       others' sums and boundary slices in an iteration, about
+ *                       that many ms; then the solve ends with HOL_ETIMEOUT
+ *                       (0: at once; 0..10000, default 1000). The blocks also
+ *                       meet at hardware cluster barriers, which have no limit of
+ *                       their own: each block reaches them because its waits end
  *   "persistent_cg"     plain mixed CG chunks in one cooperative launch (0/1)
  *   "pdl"               programmatic dependent launch of the CG iteration
  *                       kernels: each may be scheduled while its predecessor

@@ -872,8 +872,7 @@ static int cg_run_resident(hol_ctx* c, const double* b, double* v, int n_rhs, co
         all &= ih[2 * R + k];
     }
     const int* g = ih + 4 * R;
-    if (g[DCG_ERR])
-        return set_error(HOL_ENUMERIC, "cg_solve: non-finite residual (rhs %d)", g[DCG_ERR_RHS]);
+    if (g[DCG_ERR]) return dcg_error("cg_solve", g);
     if (!all)
         return set_error(HOL_ENOTCONV, "cg_solve: not converged within %d iterations", o->max_iter);
     return HOL_OK;

@@ -310,6 +310,7 @@ extern "C" int hol_create(const hol_params* p, hol_ctx** out)
     c->merged = 0;
     c->fused = 0;
     c->resident = c->exact ? 0 : 1;
+    c->resident_wait = 1000;
     c->pdl = 1;
     c->kpm_a1 = 1.0;
     c->kpm_a2 = 1.0;
@@ -591,6 +592,10 @@ extern "C" int hol_set_option(hol_ctx* c, const char* name, int value)
         if (value && c->exact)
             return set_error(HOL_EINVAL, "hol_set_option: resident_cg is checkerboard only");
         c->resident = value ? 1 : 0;
+    } else if (is("resident_wait_ms")) {
+        if (value < 0 || value > 10000)
+            return set_error(HOL_EINVAL, "hol_set_option: resident_wait_ms must be 0..10000");
+        c->resident_wait = value;
     } else if (is("pdl")) {
         c->pdl = value ? 1 : 0;
     } else if (is("fused_pc_update")) {
@@ -642,6 +647,7 @@ extern "C" int hol_get_option(const hol_ctx* c, const char* name, int* value)
     else if (is("merged_cg")) *value = c->merged;
     else if (is("fused_cg")) *value = c->fused;
     else if (is("resident_cg")) *value = c->resident;
+    else if (is("resident_wait_ms")) *value = c->resident_wait;
     else if (is("pdl")) *value = c->pdl;
     else if (is("scalar_handoff")) *value = c->handoff;
     else if (is("kpm_queue")) *value = c->kpm_queue;

@@ -160,9 +160,7 @@ extern "C" int cg_solve_graph(hol_ctx* c, const double* b, double* v, int n_rhs,
         all &= ih[n_rhs + k];
     }
     const int* gs = ih.data() + 3 * n_rhs;
-    if (gs[DCG_ERR])
-        return set_error(HOL_ENUMERIC, "cg_solve_graph: non-finite residual (rhs %d)",
-                         gs[DCG_ERR_RHS]);
+    if (gs[DCG_ERR]) return dcg_error("cg_solve_graph", gs);
     if (!all)
         return set_error(HOL_ENOTCONV, "cg_solve_graph: not converged within %d iterations",
                          o->max_iter);
@@ -252,8 +250,7 @@ extern "C" int hmc_batch_graph(hol_ctx* const* ctxs, int n_chains, double* const
     if (bad != HOL_OK) {
         HOL_CUDA(cudaEventRecord(st.e[0], os));
         HOL_CUDA(cudaStreamWaitEvent(user, st.e[0], 0));
-        return set_error(bad, "hmc_batch_graph: a solve of chain %d %s", bad_k,
-                         bad == HOL_ENUMERIC ? "met a non-finite residual" : "did not converge");
+        return set_error(bad, "hmc_batch_graph: a solve of chain %d %s", bad_k, dcg_failure(bad));
     }
     for (int k = 0; k < n_chains; ++k) {
         const double* hk = h.data() + 6 * k;
@@ -332,7 +329,7 @@ extern "C" int measure_batch_graph(hol_ctx* const* ctxs, int n_chains, const dou
         const int bad = gs[DCG_COUNT * k + DCG_STICKY];
         if (bad)
             return set_error(bad, "measure_batch_graph: a probe solve of chain %d %s", k,
-                             bad == HOL_ENUMERIC ? "met a non-finite residual" : "did not converge");
+                             dcg_failure(bad));
     }
     return HOL_OK;
 }

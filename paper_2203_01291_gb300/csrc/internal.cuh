@@ -268,6 +268,7 @@ struct hol_ctx {
     int pc_fuse;             // PCG: vector update fused into the preconditioner's transform
     int* field_cnt;          // finished-block counts of k_field and k_force_bands (zero between launches)
     int resident;            // launch option "resident_cg": plain CG with its state on chip
+    int resident_wait;       // launch option "resident_wait_ms": longest wait between its blocks
     hol::ResPlan res_plan[2];    // its plan for the last n_rhs, by precision (resident.cu)
 };
 
@@ -402,6 +403,19 @@ struct DcgState {
 inline size_t dcg_bytes(long R)
 {
     return (size_t)(4 * R) * sizeof(double) + (size_t)(4 * R + DCG_COUNT) * sizeof(int);
+}
+// Message and code of a failed solve from its g[DCG_ERR].
+inline int dcg_error(const char* fn, const int* g)
+{
+    if (g[DCG_ERR] == HOL_ETIMEOUT)
+        return set_error(HOL_ETIMEOUT, "%s: a wait between the blocks of a cluster ran out (rhs %d)", fn,
+                         g[DCG_ERR_RHS]);
+    return set_error(HOL_ENUMERIC, "%s: non-finite residual (rhs %d)", fn, g[DCG_ERR_RHS]);
+}
+inline const char* dcg_failure(int code)
+{
+    return code == HOL_ETIMEOUT   ? "waited too long for a block of its cluster"
+           : code == HOL_ENUMERIC ? "met a non-finite residual" : "did not converge";
 }
 inline DcgState dcg_state(const hol_ctx* c)
 {

@@ -146,6 +146,7 @@ int resident_enqueue(hol_ctx* c, const double* b, double* v, int n_rhs, const ho
     a.rel_every = (!f64 && o->reliable_every > 0) ? o->reliable_every : 1 << 30;
     a.slots = p.slots;
     a.tm_cols = p.tm_cols;
+    a.wait_tries = (int)((long)c->resident_wait * 1000000L / kMbTryNs);
     a.tol = o->tol;
     a.th = c->th;
     a.d = dcg_state(c);

@@ -65,6 +65,7 @@ struct ResArgs {
     int T, n_rhs, max_iter, chk, rel_every;
     int slots;             // most slices of one block
     int tm_cols;           // tensor-memory columns (TM instances)
+    int wait_tries;        // of a wait for the other blocks (mb_wait)
     double tol, th;
     DcgState d;
 };
@@ -295,8 +296,12 @@ __device__ __forceinline__ void tm_st(unsigned a, const float (&p)[N])
 // shared memories; both complete on a barrier of the receiving block, whose wait
 // is the only one (a cluster barrier costs a fence of everything before it, some
 // thousand cycles, each time). Two barriers take turns: a block two exchanges
-// ahead of another cannot exist, one ahead can. The wait is bounded; a cluster's
-// blocks are resident together, so it only ever ends by completion.
+// ahead of another cannot exist, one ahead can. A cluster's blocks are resident
+// together, so a wait ends by completion; it is bounded all the same (wait_tries of
+// kMbTryNs each). A block whose wait runs out waits once more, kMbDrain tries, for the
+// copies on their way to it, and ends its segment; the others then run out of theirs,
+// so every block reaches the cluster barriers that follow, and the solve ends
+// with HOL_ETIMEOUT.
 __device__ __forceinline__ unsigned sm_addr(const void* p)
 {
     return (unsigned)__cvta_generic_to_shared(p);
@@ -333,16 +338,17 @@ __device__ __forceinline__ void st_async8(unsigned dst, T8 v, unsigned mb)
                  "l"(u), "r"(mb)
                  : "memory");
 }
-constexpr int kMbTries = 1 << 16;   // each waits up to a hardware time limit
-__device__ __forceinline__ bool mb_wait(unsigned mb, int parity)
+constexpr int kMbTryNs = 20000;
+constexpr int kMbDrain = 50000;     // one second
+__device__ __forceinline__ bool mb_wait(unsigned mb, int parity, int tries)
 {
-    for (int k = 0; k < kMbTries; ++k) {
+    for (int k = 0; k < tries; ++k) {
         int ok;
         asm volatile("{\n.reg .pred p;\n"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n"
                      "selp.b32 %0, 1, 0, p;\n}\n"
                      : "=r"(ok)
-                     : "r"(mb), "r"(parity)
+                     : "r"(mb), "r"(parity), "r"(kMbTryNs)
                      : "memory");
         if (ok) return true;
     }
@@ -493,6 +499,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
     __shared__ int s_stop;                // 1: end of the segment, 2: not finite
     __shared__ __align__(8) unsigned long long s_mb[2];
     __shared__ int s_item;
+    __shared__ int s_lost;                // a wait of some block of the cluster ran out
     // |b|, (tol |b|)^2 on the scale of r, the exponent of |b| (pow2_hi): of the item in
     // hand, here and not in registers of the iteration
     __shared__ double s_bnorm, s_limit;
@@ -620,8 +627,9 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
     // slots than the barrier it saves.
     int par = 0;
     if (threadIdx.x < 2) mb_init(sm_addr(&s_mb[threadIdx.x]), 1);
+    if (threadIdx.x == 0) s_lost = 0;
     cl.sync();
-    bool lost = false;      // a wait ran out (never in a working cluster)
+    bool lost = false;      // a wait of this block ran out (warp 0; never in a working cluster)
     unsigned mbk = 0;       // exchanges so far: barrier mbk & 1, its phase mbk >> 1
     auto half_sum = [&](AT v) {
 #pragma unroll
@@ -642,7 +650,12 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 if (l16 < cs)
                     st_async8(sm_remote(sm_addr(&red_c[par][which][crank]), l16), v,
                               sm_remote(mb, l16));
-                if (!lost) lost = !mb_wait(mb, (int)(mbk >> 1) & 1);
+                const int phase = (int)(mbk >> 1) & 1;
+                if (!mb_wait(mb, phase, a.wait_tries)) {
+                    lost = true;
+                    mb_wait(mb, phase, kMbDrain);
+                }
+                __syncwarp();
                 v = half_sum(l16 < cs ? red_c[par][which][l16] : A::zero());
             }
             const AT o = A::shfl(v, 16);
@@ -788,9 +801,10 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         return acc;
     };
 
-    // the failure flags of the solve: of several clusters' failures a number that is not
-    // finite counts over a missed tolerance, whichever comes last
-    static_assert(HOL_ENUMERIC < HOL_ENOTCONV && HOL_ENOTCONV < 0, "the code that counts is the lower one");
+    // the failure flags of the solve: of several clusters' failures the code that counts
+    // is a timeout, then a number that is not finite, then a missed tolerance, whichever
+    // comes last (the codes fall in that order)
+    static_assert(HOL_ETIMEOUT < HOL_ENUMERIC && HOL_ENUMERIC < HOL_ENOTCONV && HOL_ENOTCONV < 0, "order");
     auto fail = [&](int code, int rhs) {
         if (code != HOL_ENOTCONV) {
             a.d.g[DCG_ERR_RHS] = rhs;   // one failing rhs (any); reported only
@@ -1030,8 +1044,9 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 // the next check_every iterations in flight when it reads this, so a solution
                 // that stops here at once is further from the exact one (1.05 to 1.5 times
                 // on average, at L = 32 to 4)
-                int stop = lost ? 2 : 0;
-                if (!lost && since > 0 && since % a.chk == 0) {
+                const bool out = __any_sync(kFull, lost);
+                int stop = out ? 2 : 0;
+                if (!out && since > 0 && since % a.chk == 0) {
                     stop = A::stop(gamma, s_limit);
                     const bool first = stop == 1 && !below;
                     below = first;
@@ -1115,6 +1130,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         // ------------------------------------------------ fold and true residual
         // every block has read its exchange slots and s: the FP64 exchange takes
         // their place. v += x, C v to the successor
+        if (wid == 0 && __any_sync(kFull, lost) && lane < cs) *cl.map_shared_rank(&s_lost, lane) = 1;
         cl.sync();
         const double down = pow2_hi(0u - s_bxs);
         double* const ex64_next0 = cl.map_shared_rank(ex64, next);
@@ -1230,7 +1246,8 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
 #pragma unroll
         for (int k = 0; k < K; ++k) halo_recv(k, hpar, r[k], false);
         hpar ^= 1;
-        bad = bad || !isfinite(tres);
+        const bool timeout = s_lost != 0;
+        bad = bad || timeout || !isfinite(tres);
         if (bad || tres < a.tol || it >= a.max_iter) {
             const unsigned bxs = s_bxs;
             if (bxs != 0)   // v on the scale of b
@@ -1253,9 +1270,13 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 a.d.tres[item] = tres;
                 a.d.done[item] = ok;
                 a.d.rstate[item] = RS_DONE;
-                if (!ok) fail(bad ? HOL_ENUMERIC : HOL_ENOTCONV, item);
+                if (!ok) fail(timeout ? HOL_ETIMEOUT : bad ? HOL_ENUMERIC : HOL_ENOTCONV, item);
             }
             item = -1;
+        }
+        if (timeout) {   // uniform over the cluster; its exchanges are no longer in step
+            cl.sync();   // the neighbours have read this block's slots
+            break;
         }
     }
     if constexpr (TM) {
