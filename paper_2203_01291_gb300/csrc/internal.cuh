@@ -155,15 +155,20 @@ struct KpmPlan {
 };
 
 struct ResArgs;
-// Launch plan of the on-chip CG for n_rhs right-hand sides (resident.cu).
+// Launch plan of the on-chip CG (resident.cu).
 struct ResPlan {
-    int n_rhs;           // 0: not yet planned
-    int cs, clusters;    // blocks per cluster; clusters launched
+    int cs, clusters;    // blocks per cluster; clusters launched (in a table: resident at once)
     int warps, k, slots; // warps per block, slices per lane group, most slices per block
     int tm_cols;         // tensor-memory columns (0: none used)
     size_t smem;
-    double us;           // modelled time of one iteration of all right-hand sides
+    double us;           // modelled time of one iteration of all right-hand sides (in a table: of one)
     void (*fn)(ResArgs); // null: no plan fits
+};
+// The plans of one precision: at most 16 cluster sizes, without and with tensor memory.
+struct ResTable {
+    int n;               // plans in p
+    int built;
+    ResPlan p[32];
 };
 
 }  // namespace hol
@@ -269,7 +274,7 @@ struct hol_ctx {
     int* field_cnt;          // finished-block counts of k_field and k_force_bands (zero between launches)
     int resident;            // launch option "resident_cg": plain CG with its state on chip
     int resident_wait;       // launch option "resident_wait_ms": longest wait between its blocks
-    hol::ResPlan res_plan[2];    // its plan for the last n_rhs, by precision (resident.cu)
+    hol::ResTable res_table[2];  // its launch plans, by precision (resident.cu)
 };
 
 namespace hol {
@@ -444,7 +449,7 @@ int cg_run_dev(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_o
 // The plain CG with its state on chip (resident.cu): whether the context and
 // options take it for n_rhs right-hand sides, and one solve enqueued on s
 // (capturable; results in dcg_state(c)).
-const ResPlan& resident_plan(hol_ctx* c, int prec, int n_rhs);
+ResPlan resident_plan(hol_ctx* c, int prec, int n_rhs);
 bool resident_ok(hol_ctx* c, const hol_cg_opts* o, int n_rhs);
 int resident_enqueue(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_opts* o,
                      cudaStream_t s);

@@ -40,22 +40,20 @@ int launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[1], const R
 
 }  // namespace
 
-// Cluster size and register sets for n_rhs right-hand sides: the smallest
-// modelled time of one iteration of all of them,
-//   max(1, n_rhs / resident clusters) * (latency + values per block * rate).
-const ResPlan& resident_plan(hol_ctx* c, int prec, int n_rhs)
+// Every cluster size and register set that fits, with the clusters the device
+// holds at once: asked of the driver once per context and precision, since a
+// program may solve for another number of right-hand sides at every call (the
+// questions, ten to thirty of each kind, took as long as a small solve).
+static void build_table(hol_ctx* c, int prec)
 {
-    ResPlan& best = c->res_plan[prec == HOL_F64 ? 1 : 0];
-    if (best.n_rhs == n_rhs) return best;
-    best = ResPlan{};
-    best.n_rhs = n_rhs;
-    if (c->exact) return best;
+    ResTable& tab = c->res_table[prec == HOL_F64 ? 1 : 0];
+    tab.n = 0;
+    tab.built = 1;
+    if (c->exact) return;
     const size_t w = prec == HOL_F64 ? 8 : 4;
-    double t_best = 1e30;
     for (int cs = 1; cs <= kMaxCluster && cs <= c->T; ++cs)
         for (int tm = 0; tm < 2; ++tm) {
             ResPlan p{};
-            p.n_rhs = n_rhs;
             p.cs = cs;
             p.slots = (c->T + cs - 1) / cs;
             ResKernel k{};
@@ -68,6 +66,7 @@ const ResPlan& resident_plan(hol_ctx* c, int prec, int n_rhs)
                 k.fn = nullptr;
             }
             if (!k.fn) continue;
+            p.fn = k.fn;
             p.smem = (size_t)((tm ? 2 : 4) * p.slots + 11) * k.sl * w;
             if (tm) {
                 // p, x and s D: three windows of K E columns, four warps side by side
@@ -79,40 +78,53 @@ const ResPlan& resident_plan(hol_ctx* c, int prec, int n_rhs)
             if (p.smem > kResSmem) continue;
             if (cs > 8 && cudaFuncSetAttribute((const void*)k.fn,
                                                cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                              cudaSuccess)
+                              cudaSuccess) {
+                cudaGetLastError();
                 continue;
+            }
             if (smem_raise((const void*)k.fn, p.smem) != HOL_OK) continue;
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute at[1];
             launch_config(cfg, at, p, 1, nullptr);
-            int nc = 0;
-            if (cudaOccupancyMaxActiveClusters(&nc, (const void*)k.fn, &cfg) != cudaSuccess ||
-                nc < 1) {
+            if (cudaOccupancyMaxActiveClusters(&p.clusters, (const void*)k.fn, &cfg) != cudaSuccess ||
+                p.clusters < 1) {
                 cudaGetLastError();
                 continue;
             }
-            p.clusters = std::min(nc, n_rhs);
             // measured (us): the block barriers and the scalar chain; the
             // exchange across blocks; a lane's own chain; the block's bandwidth
             const double vals = (double)(p.slots + 2) * c->N, ke = p.k * k.e;
-            const double us = prec == HOL_F64
-                                  ? 3.5 + (cs > 1 ? 0.5 : 0.0) + 0.4 * ke + vals * 0.0035
-                                  : 1.3 + (cs > 1 ? 0.3 : 0.0) + ke * (tm ? 0.06 : 0.13) + vals * 0.00025;
-            const double t = std::max(1.0, (double)n_rhs / nc) * us;
-            if (t < t_best) {
-                t_best = t;
-                best = p;
-                best.fn = k.fn;
-            }
+            p.us = prec == HOL_F64 ? 3.5 + (cs > 1 ? 0.5 : 0.0) + 0.4 * ke + vals * 0.0035
+                                   : 1.3 + (cs > 1 ? 0.3 : 0.0) + ke * (tm ? 0.06 : 0.13) + vals * 0.00025;
+            tab.p[tab.n++] = p;
         }
-    best.us = t_best;
+}
+
+// The plan for n_rhs right-hand sides: the smallest modelled time of one
+// iteration of all of them,
+//   max(1, n_rhs / resident clusters) * (latency + values per block * rate).
+ResPlan resident_plan(hol_ctx* c, int prec, int n_rhs)
+{
+    const ResTable& tab = c->res_table[prec == HOL_F64 ? 1 : 0];
+    if (!tab.built) build_table(c, prec);
+    ResPlan best{};
+    best.us = 1e30;
+    for (int k = 0; k < tab.n; ++k) {
+        const ResPlan& p = tab.p[k];
+        const double us = std::max(1.0, (double)n_rhs / p.clusters) * p.us;
+        if (us < best.us) {
+            best = p;
+            best.us = us;
+        }
+    }
+    best.clusters = std::min(best.clusters, n_rhs);
     return best;
 }
 
 bool resident_ok(hol_ctx* c, const hol_cg_opts* o, int n_rhs)
 {
     if (!c->resident || c->exact || o->precond || c->fused || c->merged || c->persist) return false;
-    const ResPlan& p = resident_plan(c, o->prec, n_rhs);
+    const ResPlan p = resident_plan(c, o->prec, n_rhs);
     if (!p.fn) return false;
     if (o->prec == HOL_F64) {
         // bound by the FP64 pipes of the clusters' multiprocessors, where the
@@ -129,7 +141,7 @@ bool resident_ok(hol_ctx* c, const hol_cg_opts* o, int n_rhs)
 int resident_enqueue(hol_ctx* c, const double* b, double* v, int n_rhs, const hol_cg_opts* o,
                      cudaStream_t s)
 {
-    const ResPlan& p = resident_plan(c, o->prec, n_rhs);
+    const ResPlan p = resident_plan(c, o->prec, n_rhs);
     const bool f64 = o->prec == HOL_F64;
     ResArgs a;
     a.b = b;
