@@ -1,4 +1,4 @@
-// Shared-memory mixed-radix FFT along tau (Stockham passes of radix 4, 2, 3,
+// Shared-memory mixed-radix FFT along tau (Stockham passes of radix 8, 4, 2, 3,
 // 5, 7) over tiles of TS columns, plus complex helpers. Used by the
 // preconditioner (twisted transforms), the Fourier-accelerated leapfrog (mass
 // matrix along tau) and the measurements.
@@ -42,6 +42,30 @@ struct RadixPlan {
     int n;
     int r[16];
 };
+
+// Radix plan of a length: factors 4 first, then 2, 3, 5, 7; n = -1 if another
+// prime factor remains. fp32: an odd power of two from 8 on takes one radix 8
+// pass in place of a 4 and a 2 (a pass costs a barrier and a trip through shared
+// memory, some 200 cycles). FP64 passes are bound by the FP64 pipe and spread over
+// more warps with the smaller radices.
+__host__ __device__ constexpr RadixPlan plan_of(int T, bool fp32 = false)
+{
+    RadixPlan p{0, {}};
+    int t = T, e2 = 0;
+    for (int u = T; u % 2 == 0; u /= 2) ++e2;
+    if (fp32 && e2 >= 3 && e2 % 2 == 1) {
+        p.r[p.n++] = 8;
+        t /= 8;
+    }
+    const int rs[5] = {4, 2, 3, 5, 7};
+    for (int k = 0; k < 5; ++k)
+        while (t % rs[k] == 0 && p.n < 16) {
+            p.r[p.n++] = rs[k];
+            t /= rs[k];
+        }
+    if (t != 1) p.n = -1;
+    return p;
+}
 
 // twiddle w2[k] = exp(-i pi k / T), 0 <= k < 2T (every caller's index is in
 // range: 2 r k T / (Ns RAD) < 2T and 2 e T / RAD < 2T)
@@ -143,13 +167,16 @@ __device__ __forceinline__ void dft_small(typename Cx<R>::T2 (&a)[RAD],
 // Butterfly j (0 <= j < T/RAD) with k = j mod Ns reads in[j + r T/RAD],
 // scales input r by exp(-2 pi i r k / (Ns RAD)), takes the length-RAD DFT
 // and writes out[(j / Ns) Ns RAD + k + q Ns]. blockDim.x must be a multiple
-// of TS; (k, j / Ns) are advanced incrementally instead of divided.
-template <typename R, int RAD>
-__device__ void stockham_pass(const typename Cx<R>::T2* __restrict__ in,
-                              typename Cx<R>::T2* __restrict__ out,
-                              const typename Cx<R>::T2* __restrict__ w2, int T, int TS, int Ns)
+// of TS; (k, j / Ns) are advanced incrementally instead of divided. TSC > 0: TS
+// at compile time.
+template <typename R, int RAD, int TSC>
+__device__ __forceinline__ void stockham_pass(const typename Cx<R>::T2* __restrict__ in,
+                                              typename Cx<R>::T2* __restrict__ out,
+                                              const typename Cx<R>::T2* __restrict__ w2, int T, int TS_,
+                                              int Ns)
 {
     using C2 = typename Cx<R>::T2;
+    const int TS = TSC > 0 ? TSC : TS_;
     const int nb = T / RAD;
     const int c = threadIdx.x % TS;
     const int sj = blockDim.x / TS;         // step of j per iteration
@@ -159,7 +186,7 @@ __device__ void stockham_pass(const typename Cx<R>::T2* __restrict__ in,
     const int tstep = T / (Ns * RAD);       // twiddle index step per unit of k, halved
     C2 root[RAD];                           // exp(-2 pi i e / RAD)
 #pragma unroll
-    for (int e = 0; e < RAD; ++e) root[e] = w2[2L * e * (T / RAD)];
+    for (int e = 0; e < RAD; ++e) root[e] = w2[2 * e * (T / RAD)];
     for (; j < nb; j += sj) {
         C2 a[RAD];
         a[0] = in[j * TS + c];
@@ -167,7 +194,7 @@ __device__ void stockham_pass(const typename Cx<R>::T2* __restrict__ in,
 #pragma unroll
         for (int r = 1; r < RAD; ++r) {
             const C2 v = in[(j + r * nb) * TS + c];
-            a[r] = k > 0 ? cmul(v, w2[2L * r * k * tstep]) : v;
+            a[r] = k > 0 ? cmul(v, w2[2 * r * k * tstep]) : v;
         }
         dft_small<R, RAD>(a, root);
         const int ob = jb * Ns * RAD + k;
@@ -184,7 +211,7 @@ __device__ void stockham_pass(const typename Cx<R>::T2* __restrict__ in,
 
 // Full forward DFT of length T along the first index of buf (TS columns);
 // returns the buffer holding the result.
-template <typename R>
+template <typename R, int TSC = 0>
 __device__ typename Cx<R>::T2* fft_tau(typename Cx<R>::T2* a, typename Cx<R>::T2* b,
                                        const typename Cx<R>::T2* __restrict__ w2, int T, int TS,
                                        const RadixPlan& plan)
@@ -193,11 +220,14 @@ __device__ typename Cx<R>::T2* fft_tau(typename Cx<R>::T2* a, typename Cx<R>::T2
     for (int s = 0; s < plan.n; ++s) {
         __syncthreads();
         switch (plan.r[s]) {
-        case 2: stockham_pass<R, 2>(a, b, w2, T, TS, Ns); break;
-        case 3: stockham_pass<R, 3>(a, b, w2, T, TS, Ns); break;
-        case 4: stockham_pass<R, 4>(a, b, w2, T, TS, Ns); break;
-        case 5: stockham_pass<R, 5>(a, b, w2, T, TS, Ns); break;
-        default: stockham_pass<R, 7>(a, b, w2, T, TS, Ns); break;
+        case 2: stockham_pass<R, 2, TSC>(a, b, w2, T, TS, Ns); break;
+        case 3: stockham_pass<R, 3, TSC>(a, b, w2, T, TS, Ns); break;
+        case 4: stockham_pass<R, 4, TSC>(a, b, w2, T, TS, Ns); break;
+        case 5: stockham_pass<R, 5, TSC>(a, b, w2, T, TS, Ns); break;
+        case 8:
+            if constexpr (sizeof(R) == 4) stockham_pass<R, 8, TSC>(a, b, w2, T, TS, Ns);
+            break;
+        default: stockham_pass<R, 7, TSC>(a, b, w2, T, TS, Ns); break;
         }
         Ns *= plan.r[s];
         typename Cx<R>::T2* t = a;
@@ -213,36 +243,8 @@ __device__ typename Cx<R>::T2* fft_tau(typename Cx<R>::T2* a, typename Cx<R>::T2
 // The same transform with the length T, the tile width TS and the block size
 // NT known at compile time (the lengths of the configured workloads): the
 // plan, the butterfly loops and every index division are resolved by the
-// compiler. Twiddles as in fft_tau, from shared memory.
+// compiler. The passes and twiddles are fft_tau's.
 // ---------------------------------------------------------------------------
-struct PlanCT {
-    int n;
-    int r[16];
-};
-
-// FP32: an odd power of two from 8 on takes one radix 8 pass in place of a 4 and
-// a 2 (a pass costs a barrier and a trip through shared memory, some 200
-// cycles). FP64 passes are bound by the FP64 pipe and spread over more warps
-// with the smaller radices.
-__host__ __device__ constexpr PlanCT plan_ct(int T, bool fp32)
-{
-    PlanCT p{0, {}};
-    int t = T, e2 = 0;
-    for (int u = T; u % 2 == 0; u /= 2) ++e2;
-    if (fp32 && e2 >= 3 && e2 % 2 == 1) {
-        p.r[p.n++] = 8;
-        t /= 8;
-    }
-    const int rs[5] = {4, 2, 3, 5, 7};
-    for (int k = 0; k < 5; ++k)
-        while (t % rs[k] == 0 && p.n < 16) {
-            p.r[p.n++] = rs[k];
-            t /= rs[k];
-        }
-    if (t != 1) p.n = -1;
-    return p;
-}
-
 template <typename R, int RAD, int T, int TS, int NT, int Ns>
 __device__ __forceinline__ void stockham_pass_ct(const typename Cx<R>::T2* __restrict__ in,
                                                  typename Cx<R>::T2* __restrict__ out,
@@ -282,7 +284,7 @@ __device__ __forceinline__ typename Cx<R>::T2* fft_tau_ct(typename Cx<R>::T2* a,
                                                           typename Cx<R>::T2* b,
                                                           const typename Cx<R>::T2* __restrict__ w2)
 {
-    constexpr PlanCT P = plan_ct(T, sizeof(R) == 4);
+    constexpr RadixPlan P = plan_of(T, sizeof(R) == 4);
     static_assert(P.n > 0, "length with a prime factor above 7");
     if constexpr (S < P.n) {
         constexpr int RAD = P.r[S];
@@ -293,23 +295,6 @@ __device__ __forceinline__ typename Cx<R>::T2* fft_tau_ct(typename Cx<R>::T2* a,
         __syncthreads();
         return a;
     }
-}
-
-// radix plan of a length (host): factors 4 first, then 2, 3, 5, 7; n = -1 if
-// another prime factor remains
-inline RadixPlan plan_of(int T)
-{
-    RadixPlan p;
-    p.n = 0;
-    int t = T;
-    const int rs[5] = {4, 2, 3, 5, 7};
-    for (int k = 0; k < 5; ++k)
-        while (t % rs[k] == 0 && p.n < 16) {
-            p.r[p.n++] = rs[k];
-            t /= rs[k];
-        }
-    if (t != 1) p.n = -1;
-    return p;
 }
 
 }  // namespace fft

@@ -109,6 +109,11 @@ __device__ __forceinline__ void st_cpair(double2* p, double2 a, double2 b)
 // P^{-1} P^{-T}, L = 16, Ltau = 160, 2 rhs: 15.2 -> 14.2 us; L = 32, Ltau = 200,
 // 16 rhs: 48.4 -> 40; a preconditioned iteration at L = 16, Ltau = 160, 2 rhs, all
 // kernels: 27.6 -> 24.5 us (22.5 with the paired sums of alpha and beta, cb.cuh).
+// That holds at every length: with twiddles, radix 8 and tile width taken so without
+// a compile-time length too, L = 32, 16 rhs, Ltau = 96 / 144 / 192: 39.7 / 48.9 / 58.0 -> 30.2 /
+// 44.2 / 50.4 us in FP32, 351 / 469 / 608 -> 305 / 458 / 596 in FP64; L = 16, 2 rhs, Ltau = 144:
+// 18.7 -> 16.4. What remains against the compile-time lengths (Ltau = 160: 31.7) is
+// the run-time plan: divisions by Ltau / radix and a switch per pass.
 template <bool EARLY>
 struct PdlTriggerFp32 {
     __device__ __forceinline__ PdlTriggerFp32() { if (EARLY) pdl_trigger(); }
@@ -125,32 +130,33 @@ struct PdlTriggerFp32 {
 // X_b = (Z[w] - conj Z[T-1-w]) / (2 i).
 //
 // v (real [nr][T][N]) -> vh (complex [nr][T/2][N]) = U v restricted to omega < T/2
-// TC, TSC > 0: length and tile width (sites) fixed at compile time
-// (fft_tau_ct); 0: taken from the arguments (fft_tau).
-template <typename R, int TC = 0, int TSC = 0>
+// TC > 0: length fixed at compile time (fft_tau_ct); 0: taken from the arguments
+// (fft_tau). TSC > 0: tile width (sites) fixed at compile time. TWS: the twiddles in
+// shared memory, behind the tile's two buffers (read from L2 in every pass they cost each
+// its latency); false where they do not fit there too.
+template <typename R, int TC, int TSC, bool TWS>
 __global__ void __launch_bounds__(256) k_tau_fwd(const R* __restrict__ v,
                                                  typename Cx<R>::T2* __restrict__ vh,
                                                  const typename Cx<R>::T2* __restrict__ w2g, int T_,
                                                  int N, int TS_, RadixPlan plan, R scale)
 {
     using C2 = typename Cx<R>::T2;
-    // the twiddles come to shared memory while the previous kernel ends (read
-    // from L2 in every pass they cost each its latency)
-    const C2* w2 = w2g;
-    if constexpr (TC > 0) {
-        __shared__ C2 tws[2 * TC];
-        for (int k = threadIdx.x; k < 2 * TC; k += 256) tws[k] = w2g[k];
-        w2 = tws;
-    }
-    pdl_wait();      // the input comes from the previous kernel of the stream
-    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
-    __syncthreads();
     const int T = TC > 0 ? TC : T_;
     const int TS = TSC > 0 ? TSC : TS_;
     const int TH = TS / 2;                 // transform columns
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2* a = reinterpret_cast<C2*>(smem_raw);
     C2* b = a + (long)T * TH;
+    // the twiddles come to shared memory while the previous kernel ends
+    const C2* w2 = w2g;
+    if constexpr (TWS) {
+        C2* tws = b + (long)T * TH;
+        for (int k = threadIdx.x; k < 2 * T; k += 256) tws[k] = w2g[k];
+        w2 = tws;
+    }
+    pdl_wait();      // the input comes from the previous kernel of the stream
+    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
+    __syncthreads();
     const int rhs = blockIdx.y;
     const int i0 = blockIdx.x * TS;
     const long base = (long)rhs * T * N;
@@ -166,7 +172,7 @@ __global__ void __launch_bounds__(256) k_tau_fwd(const R* __restrict__ v,
     if constexpr (TC > 0)
         res = fft_tau_ct<R, TC, TSC / 2, 256>(a, b, w2);
     else
-        res = fft_tau<R>(a, b, w2, T, TH, plan);
+        res = fft_tau<R, TSC / 2>(a, b, w2, T, TH, plan);
     const int Th = T / 2;
     const long ob = (long)rhs * Th * N;
     const R hs = R(0.5) * scale;
@@ -205,7 +211,7 @@ struct PcUpdK {
     int fold;
 };
 
-template <typename R, int TC = 0, int TSC = 0>
+template <typename R, int TC, int TSC, bool TWS>
 __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
                                                      typename Cx<R>::T2* __restrict__ vh,
                                                      const typename Cx<R>::T2* __restrict__ w2g,
@@ -218,22 +224,21 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
     // FP64 division that would otherwise precede the loads' latency. In FP64 more
     // than one costs registers and gains nothing.
     constexpr int kUpdItems = sizeof(R) == 4 ? 4 : 1;
-    // the twiddles come to shared memory while the previous kernel ends (read
-    // from L2 in every pass they cost each its latency)
-    const C2* w2 = w2g;
-    if constexpr (TC > 0) {
-        __shared__ C2 tws[2 * TC];
-        for (int k = threadIdx.x; k < 2 * TC; k += 256) tws[k] = w2g[k];
-        w2 = tws;
-    }
-    pdl_wait();      // p, q and the partials come from the previous kernel of the stream
-    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
     const int T = TC > 0 ? TC : T_;
     const int TS = TSC > 0 ? TSC : TS_;
     const int TH = TS / 2;                 // transform columns
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2* a = reinterpret_cast<C2*>(smem_raw);
     C2* b = a + (long)T * TH;
+    // the twiddles come to shared memory while the previous kernel ends
+    const C2* w2 = w2g;
+    if constexpr (TWS) {
+        C2* tws = b + (long)T * TH;
+        for (int k = threadIdx.x; k < 2 * T; k += 256) tws[k] = w2g[k];
+        w2 = tws;
+    }
+    pdl_wait();      // p, q and the partials come from the previous kernel of the stream
+    const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
     const int rhs = blockIdx.y;
     const int i0 = blockIdx.x * TS;
     const long base = (long)rhs * T * N;
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
     if constexpr (TC > 0)
         res = fft_tau_ct<R, TC, TSC / 2, 256>(a, b, w2);
     else
-        res = fft_tau<R>(a, b, w2, T, TH, plan);
+        res = fft_tau<R, TSC / 2>(a, b, w2, T, TH, plan);
     const int Th = T / 2;
     const long ob = (long)rhs * Th * N;
     const R hs = R(0.5) * scale;
@@ -352,7 +357,7 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
 // y_a + i y_b = (1 / sqrt T) conj(t_tau F_tau).
 // yh (complex [nr][T/2][N]) -> y (real [nr][T][N]); optional dot partials
 // sum(y * rdot) per (rhs, tile). `scale` is 2 / sqrt T.
-template <typename R, int TC = 0, int TSC = 0>
+template <typename R, int TC, int TSC, bool TWS>
 __global__ void __launch_bounds__(256) k_tau_inv(const typename Cx<R>::T2* __restrict__ yh,
                                                  R* __restrict__ y,
                                                  const typename Cx<R>::T2* __restrict__ w2g, int T_,
@@ -361,22 +366,21 @@ __global__ void __launch_bounds__(256) k_tau_inv(const typename Cx<R>::T2* __res
                                                  double* __restrict__ dot_part)
 {
     using C2 = typename Cx<R>::T2;
-    // the twiddles come to shared memory while the previous kernel ends (read
-    // from L2 in every pass they cost each its latency)
+    const int T = TC > 0 ? TC : T_;
+    const int TS = TSC > 0 ? TSC : TS_;
+    const int TH = TS / 2;                 // transform columns
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C2* a = reinterpret_cast<C2*>(smem_raw);
+    C2* b = a + (long)T * TH;
+    // the twiddles come to shared memory while the previous kernel ends
     const C2* w2 = w2g;
-    if constexpr (TC > 0) {
-        __shared__ C2 tws[2 * TC];
-        for (int k = threadIdx.x; k < 2 * TC; k += 256) tws[k] = w2g[k];
+    if constexpr (TWS) {
+        C2* tws = b + (long)T * TH;
+        for (int k = threadIdx.x; k < 2 * T; k += 256) tws[k] = w2g[k];
         w2 = tws;
     }
     pdl_wait();      // the input comes from the previous kernel of the stream
     const PdlTriggerFp32<sizeof(R) == 4> pdl_trig;
-    const int T = TC > 0 ? TC : T_;
-    const int TS = TSC > 0 ? TSC : TS_;
-    const int TH = TS / 2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C2* a = reinterpret_cast<C2*>(smem_raw);
-    C2* b = a + (long)T * TH;
     const int rhs = blockIdx.y;
     const int i0 = blockIdx.x * TS;
     const int Th = T / 2;
@@ -399,7 +403,7 @@ __global__ void __launch_bounds__(256) k_tau_inv(const typename Cx<R>::T2* __res
     if constexpr (TC > 0)
         res = fft_tau_ct<R, TC, TSC / 2, 256>(a, b, w2);
     else
-        res = fft_tau<R>(a, b, w2, T, TH, plan);
+        res = fft_tau<R, TSC / 2>(a, b, w2, T, TH, plan);
     const long ob = (long)rhs * T * N;
     const R hs = R(0.5) * scale;           // 1 / sqrt T
     double acc = 0.0;
@@ -1424,6 +1428,7 @@ int tile_sites(const hol_ctx* c, int prec, int n_rhs)
     return (long)c->N * n_rhs <= 8L * small * c->sms ? small : 2 * small;
 }
 
+constexpr size_t kFftSmem = 220 * 1024;   // a tile's buffers and twiddles
 size_t fft_smem(const hol_ctx* c, int prec, int ts)
 {
     const size_t cs = prec == HOL_F64 ? sizeof(double2) : sizeof(float2);
@@ -1534,43 +1539,48 @@ int precond_run(hol_ctx* c, const R* v, R* out, int n_rhs, int mode, const R* rd
 {
     using C2 = typename Cx<R>::T2;
     const int prec = sizeof(R) == 8 ? HOL_F64 : HOL_F32;
-    const RadixPlan plan = plan_of(c->T);
+    const RadixPlan plan = plan_of(c->T, sizeof(R) == 4);
     const int TS = tile_sites(c, prec, n_rhs);
-    const size_t sm = fft_smem(c, prec, TS);
+    size_t sm = fft_smem(c, prec, TS);
     const dim3 gf(ceil_div(c->N, TS), n_rhs);
     const C2* w2 = reinterpret_cast<const C2*>(prec == HOL_F64 ? (const void*)c->tw64
                                                                 : (const void*)c->tw32);
     C2* h0 = reinterpret_cast<C2*>(c->cbuf0);
     C2* h1 = reinterpret_cast<C2*>(c->cbuf1);
     int rc;
-    // the configured lengths get transforms specialised at compile time
+    // Every length takes the tile width at compile time and its twiddles from
+    // shared memory, while these fit; the configured lengths are compiled for
+    // their length besides.
     constexpr int TSS = sizeof(R) == 8 ? 4 : 8;   // tile_sites' two choices
     using FwdK = void (*)(const R*, C2*, const C2*, int, int, int, RadixPlan, R);
     using FwdU = void (*)(R*, C2*, const C2*, int, int, int, RadixPlan, R, PcUpdK<R>);
     using InvK = void (*)(const C2*, R*, const C2*, int, int, int, RadixPlan, R, const R*, double*);
-    FwdK fwd = k_tau_fwd<R>;
-    FwdU fwdu = k_tau_fwd_upd<R>;
-    InvK inv = k_tau_inv<R>;
-#define HOL_TAU_CT(TT)                                    \
-    case TT:                                              \
-        if (TS == TSS) {                                  \
-            fwd = k_tau_fwd<R, TT, TSS>;                  \
-            fwdu = k_tau_fwd_upd<R, TT, TSS>;             \
-            inv = k_tau_inv<R, TT, TSS>;                  \
-        } else {                                          \
-            fwd = k_tau_fwd<R, TT, 2 * TSS>;              \
-            fwdu = k_tau_fwd_upd<R, TT, 2 * TSS>;         \
-            inv = k_tau_inv<R, TT, 2 * TSS>;              \
-        }                                                 \
-        break;
-    switch (c->T) {
-        HOL_TAU_CT(40)
-        HOL_TAU_CT(120)
-        HOL_TAU_CT(160)
-        HOL_TAU_CT(200)
-    default: break;
-    }
+    FwdK fwd = k_tau_fwd<R, 0, 0, false>;
+    FwdU fwdu = k_tau_fwd_upd<R, 0, 0, false>;
+    InvK inv = k_tau_inv<R, 0, 0, false>;
+    const size_t tws = 2 * (size_t)c->T * sizeof(C2);
+    if (sm + tws <= kFftSmem) {
+        sm += tws;
+#define HOL_TAU_CT(TT)                                        \
+    if (TS == TSS) {                                          \
+        fwd = k_tau_fwd<R, TT, TSS, true>;                    \
+        fwdu = k_tau_fwd_upd<R, TT, TSS, true>;               \
+        inv = k_tau_inv<R, TT, TSS, true>;                    \
+    } else {                                                  \
+        fwd = k_tau_fwd<R, TT, 2 * TSS, true>;                \
+        fwdu = k_tau_fwd_upd<R, TT, 2 * TSS, true>;           \
+        inv = k_tau_inv<R, TT, 2 * TSS, true>;                \
+    }                                                         \
+    break;
+        switch (c->T) {
+        case 40: HOL_TAU_CT(40)
+        case 120: HOL_TAU_CT(120)
+        case 160: HOL_TAU_CT(160)
+        case 200: HOL_TAU_CT(200)
+        default: HOL_TAU_CT(0)
+        }
 #undef HOL_TAU_CT
+    }
     if ((rc = set_smem_attr<R>(up ? (const void*)fwdu : (const void*)fwd, sm))) return rc;
     if ((rc = set_smem_attr<R>((const void*)inv, sm))) return rc;
     const R isq = (R)(1.0 / sqrt((double)c->T));
@@ -1682,7 +1692,7 @@ int precond_check_shape(const hol_ctx* c)
 {
     const RadixPlan p = plan_of(c->T);
     if (p.n < 0) return set_error(HOL_EINVAL, "preconditioner: Ltau=%d has a prime factor > 7", c->T);
-    if (fft_smem(c, HOL_F64, c->N < 1024 ? 8 : 16) > 220 * 1024)
+    if (fft_smem(c, HOL_F64, c->N < 1024 ? 8 : 16) > kFftSmem)
         return set_error(HOL_EINVAL, "preconditioner: Ltau=%d too long for one tile", c->T);
     if (c->N > kKpmMaxE * 256) return set_error(HOL_EINVAL, "preconditioner: N too large");
     return HOL_OK;
