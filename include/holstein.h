@@ -501,6 +501,8 @@ int hol_get_bounds(hol_ctx* ctx, double* bmin, double* bmax, void* stream);
  * slices per group, warps per block, layout (the "layout"
  * values of hol_set_option), and its time in ms. A context with the exact
  * propagator (HOL_KINETIC_EXACT) tunes the scalar layout 0 only.
+ * The choice is for the operator and the iteration kernels: a plain solve that runs on
+ * chip (resident_cg, the default) does not use it.
  * Requires hol_set_field; overwrites context scratch; synchronises `stream`.
  */
 int hol_tune(hol_ctx* ctx, int n_rhs, int* best_k, int* best_warps, int* best_vec,
@@ -509,7 +511,9 @@ int hol_tune(hol_ctx* ctx, int n_rhs, int* best_k, int* best_warps, int* best_ve
 /*
  * Runtime launch options of a context (no counterpart in the paper; results
  * are the same up to rounding whichever is chosen):
- *   "slices_per_group"  tau slices streamed per lane group (divides Ltau)
+ *   "slices_per_group"  tau slices streamed per lane group (divides Ltau). This,
+ *                       warps_per_block and layout: operator and iteration
+ *                       kernels, no effect on a solve on chip (resident_cg)
  *   "warps_per_block"   1, 2 or 4 for the operator kernels
  *   "layout"            0 scalar, 1 float4, 2 float4 with a two-slice cp.async
  *                       ring, 6 the same with a three-slice ring (2 and 6

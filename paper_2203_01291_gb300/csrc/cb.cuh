@@ -183,7 +183,8 @@ __device__ __forceinline__ double warp_sum_array(const double* __restrict__ a, i
 // latency of loads instead of two. Every operator warp of a CG iteration forms
 // beta from two such sums, and every update block alpha: a trajectory at L = 16,
 // Ltau = 160 (one such pair of sums after the other in each of its dependent
-// kernels) 375 -> 344 ms, six mixed chains 58.6 -> 55.0.
+// kernels) 375 -> 344 ms, six mixed chains 58.6 -> 55.0 (the same build 340 to 356 and
+// 55 to 56 from one machine to the next).
 __device__ __forceinline__ double2 warp_sum_pair(const double* __restrict__ a, int na,
                                                  const double* __restrict__ b, int nb)
 {

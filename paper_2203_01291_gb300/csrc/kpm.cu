@@ -7,7 +7,11 @@
 //
 // What bounds both kernels is the chain of dependent Bbar applications of omega
 // = 0 (N_P falls like 1 / (omega + 1/2), so its two series are several times
-// longer than the next); all other problems fit beside it.
+// longer than the next); all other problems fit beside it. Against the older kernels
+// (kpm_registers 0..3), P^{-1} P^{-T} at Ltau = 120 for every even L from 4 to 32 on 2 and
+// 16 right-hand sides: FP32 as fast at L = 4 and 6 (14 us, launches), else 1.04 to 2.2 times
+// as fast as the best of them; FP64 1.1 to 2.6 times. They remain for callers that
+// select them.
 //   k_kpm_strip (FP32, L <= 18): one warp per part with the slice in the strip
 //   layout (strip.cuh), so a step has no barrier: about 150 cycles a step, the
 //   latency of its shuffles and dependent multiply-adds. Steps carry the

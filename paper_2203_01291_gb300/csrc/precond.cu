@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(256) k_tau_fwd_upd(R* __restrict__ v,
                                                      R scale, PcUpdK<R> u)
 {
     using C2 = typename Cx<R>::T2;
-    // The first kUpdItems elements of a thread (FP32: all of them at the configured
-    // lengths) are loaded before alpha is formed, a chain of partial sums and an
+    // The first kUpdItems elements of a thread (FP32: all of them up to Ltau = 256 in
+    // an 8-site tile, 128 in a 16-site one) are loaded before alpha is formed, a chain of partial sums and an
     // FP64 division that would otherwise precede the loads' latency. In FP64 more
     // than one costs registers and gains nothing.
     constexpr int kUpdItems = sizeof(R) == 4 ? 4 : 1;
@@ -1688,6 +1688,8 @@ int precond_tiles(const hol_ctx* c, int prec, int n_rhs)
     return ceil_div(c->N, tile_sites(c, prec, n_rhs));
 }
 
+// The longest Ltau is that of the 8- and 16-site FP64 tiles the transforms once used
+// (twice today's): what was refused stays refused.
 int precond_check_shape(const hol_ctx* c)
 {
     const RadixPlan p = plan_of(c->T);

@@ -298,10 +298,10 @@ __device__ __forceinline__ void tm_st(unsigned a, const float (&p)[N])
 // thousand cycles, each time). Two barriers take turns: a block two exchanges
 // ahead of another cannot exist, one ahead can. A cluster's blocks are resident
 // together, so a wait ends by completion; it is bounded all the same (wait_tries of
-// kMbTryNs each). A block whose wait runs out waits once more, kMbDrain tries, for the
-// copies on their way to it, and ends its segment; the others then run out of theirs,
-// so every block reaches the cluster barriers that follow, and the solve ends
-// with HOL_ETIMEOUT.
+// kMbTryNs each). A block whose wait runs out ends its segment and waits once more,
+// kMbDrain tries, for the copies on their way to it; the others then run out of
+// their waits, so every block reaches the cluster barriers that follow, and the solve
+// ends with HOL_ETIMEOUT.
 __device__ __forceinline__ unsigned sm_addr(const void* p)
 {
     return (unsigned)__cvta_generic_to_shared(p);
@@ -353,6 +353,17 @@ __device__ __forceinline__ bool mb_wait(unsigned mb, int parity, int tries)
         if (ok) return true;
     }
     return false;
+}
+
+// After a wait that ran out: waits for what is still on its way into this block
+// (barriers mb[0], mb[1], exchanges so far n), then sets the flag in every block of the
+// cluster. Out of line: inlined, never executed, it changed the iteration's code
+// (L = 18, Ltau = 160, 8 rhs: 3.40 -> 3.66 us per iteration).
+static __device__ __noinline__ void mb_gave_up(unsigned mb, unsigned n, unsigned flag, int cs)
+{
+    if ((int)threadIdx.x >= cs) return;
+    for (unsigned x = n > 2 ? n - 2 : 0; x < n; ++x) mb_wait(mb + 8 * (x & 1), (int)(x >> 1) & 1, kMbDrain);
+    asm volatile("st.shared::cluster.u32 [%0], %1;\n" ::"r"(sm_remote(flag, threadIdx.x)), "r"(1) : "memory");
 }
 
 // A right-hand side is solved as b / 2^ex, ex the exponent of |b|, so that the FP32
@@ -496,7 +507,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
     __shared__ AT red_c[2][2][16];        // [parity][sum][block of the cluster]
     __shared__ double red64[2][16 * 16];
     __shared__ R s_step[2];               // alpha, beta
-    __shared__ int s_stop;                // 1: end of the segment, 2: not finite
+    __shared__ int s_stop;                // 1: end of the segment, 2: not finite, 3: a wait ran out
     __shared__ __align__(8) unsigned long long s_mb[2];
     __shared__ int s_item;
     __shared__ int s_lost;                // a wait of some block of the cluster ran out
@@ -627,7 +638,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
     // slots than the barrier it saves.
     int par = 0;
     if (threadIdx.x < 2) mb_init(sm_addr(&s_mb[threadIdx.x]), 1);
-    if (threadIdx.x == 0) s_lost = 0;
+    if (threadIdx.x == 0) s_stop = s_lost = 0;
     cl.sync();
     bool lost = false;      // a wait of this block ran out (warp 0; never in a working cluster)
     unsigned mbk = 0;       // exchanges so far: barrier mbk & 1, its phase mbk >> 1
@@ -650,12 +661,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 if (l16 < cs)
                     st_async8(sm_remote(sm_addr(&red_c[par][which][crank]), l16), v,
                               sm_remote(mb, l16));
-                const int phase = (int)(mbk >> 1) & 1;
-                if (!mb_wait(mb, phase, a.wait_tries)) {
-                    lost = true;
-                    mb_wait(mb, phase, kMbDrain);
-                }
-                __syncwarp();
+                if (!lost) lost = !mb_wait(mb, (int)(mbk >> 1) & 1, a.wait_tries);
                 v = half_sum(l16 < cs ? red_c[par][which][l16] : A::zero());
             }
             const AT o = A::shfl(v, 16);
@@ -820,8 +826,9 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         if (crank == 0 && wid == 0) {
             // the ready right-hand side with the fewest iterations; an
             // unfinished one in hand (left running) is given back for it
+            // (none after a wait ran out: the cluster's exchanges are no longer in step)
             int pick = -1;
-            for (int tries = 0; tries < a.n_rhs && pick < 0; ++tries) {
+            for (int tries = s_lost ? a.n_rhs : 0; tries < a.n_rhs && pick < 0; ++tries) {
                 int best = 0x7fffffff, bi = -1;
                 for (int k = lane; k < a.n_rhs; k += 32)
                     if (__ldcg(a.d.rstate + k) == RS_READY) {
@@ -1044,9 +1051,8 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 // the next check_every iterations in flight when it reads this, so a solution
                 // that stops here at once is further from the exact one (1.05 to 1.5 times
                 // on average, at L = 32 to 4)
-                const bool out = __any_sync(kFull, lost);
-                int stop = out ? 2 : 0;
-                if (!out && since > 0 && since % a.chk == 0) {
+                int stop = lost ? 3 : 0;
+                if (!lost && since > 0 && since % a.chk == 0) {
                     stop = A::stop(gamma, s_limit);
                     const bool first = stop == 1 && !below;
                     below = first;
@@ -1062,7 +1068,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
             }
             __syncthreads();
             if (s_stop) {
-                bad = s_stop == 2;
+                bad = s_stop >= 2;
                 hpar ^= 1;
                 break;
             }
@@ -1130,7 +1136,7 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
         // ------------------------------------------------ fold and true residual
         // every block has read its exchange slots and s: the FP64 exchange takes
         // their place. v += x, C v to the successor
-        if (wid == 0 && __any_sync(kFull, lost) && lane < cs) *cl.map_shared_rank(&s_lost, lane) = 1;
+        if (s_stop == 3) mb_gave_up(sm_addr(s_mb), mbk, sm_addr(&s_lost), cs);
         cl.sync();
         const double down = pow2_hi(0u - s_bxs);
         double* const ex64_next0 = cl.map_shared_rank(ex64, next);
@@ -1273,10 +1279,6 @@ __global__ void __launch_bounds__(512, 1) k_cg_resident(ResArgs a)
                 if (!ok) fail(timeout ? HOL_ETIMEOUT : bad ? HOL_ENUMERIC : HOL_ENOTCONV, item);
             }
             item = -1;
-        }
-        if (timeout) {   // uniform over the cluster; its exchanges are no longer in step
-            cl.sync();   // the neighbours have read this block's slots
-            break;
         }
     }
     if constexpr (TM) {
