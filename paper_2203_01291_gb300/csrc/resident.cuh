@@ -36,12 +36,12 @@
 //
 // Bounds and measurements (GB300, us per iteration of all right-hand sides,
 // solves to 1e-10, against the two-kernel iteration): L = 4, Ltau = 40, 1 rhs
-// 1.9 / 10.2 (a chain of block barriers and the scalar step, some 3500 cycles);
-// L = 16, Ltau = 160, 2 rhs 2.7 / 14.6; L = 28, Ltau = 120, 128 rhs 57 / 115
-// and L = 32, Ltau = 200, 16 rhs 15.1 / 30 (issue slots and shared memory of the
+// 1.5 / 8.6 (a chain of block barriers and the scalar step, some 3000 cycles);
+// L = 16, Ltau = 160, 2 rhs 2.6 / 9.8; L = 28, Ltau = 120, 128 rhs 52 / 101
+// and L = 32, Ltau = 200, 16 rhs 14.3 / 22 (issue slots and shared memory of the
 // multiprocessors that clusters of 9 and 16 blocks reach, 135 and 112 of 152; a
 // quarter of it the FP64 true residual, bound by the FP64 pipes). FP64
-// iterations, L = 4: 5.9 / 13.1.
+// iterations, L = 4: 5.5 / 11.7.
 #pragma once
 
 #include <cooperative_groups.h>
