@@ -157,7 +157,7 @@ typedef struct hol_cg_opts {
  * b, v: FP64 [n_rhs][T][N] (device). Convergence of every right-hand side is
  * certified with an FP64 true residual |b - M^T M v| / |b| < tol. With
  * opts->prec HOL_F32 the iterations run in FP32 (dot products: FP32 within a
- * group of four products, for |M p|^2 within a thread's share of a slice; the groups'
+ * group of two or four products, for |M p|^2 within a thread's share of a slice; the groups'
  * sums as compensated float pairs of some 48 bits, over blocks FP64 in the iteration
  * kernels and pairs in a solve on chip) and every reliable_every iterations, and whenever the recursive residual
  * estimate falls below tol, the FP32 increment is folded into the FP64 v and
